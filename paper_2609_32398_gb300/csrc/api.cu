@@ -71,11 +71,6 @@ do_status check_route(const Problem &p, const RouteArgs &r) {
     return DO_OK;
 }
 
-// The vector stores of the fast selection kernel want 16-byte aligned rows.
-bool route_fast_ok(const RouteArgs *r) {
-    return !r || (aligned(r->ids, 16) && aligned(r->combine, 16));
-}
-
 // Workspace of do_routing: [status word | pad to 256 B | signatures [L][E][W] |
 // dispatch scratch (route_scratch_ints)].
 size_t routing_bits_bytes(const Problem &p) {
@@ -115,14 +110,6 @@ do_status do_signatures(const float *logits, int64_t T, int32_t E, int32_t k, in
     if (!logits || !bits || !counts) return DO_ERR_INVALID_ARG;
     if (!aligned(logits, 4) || !aligned(bits, 4) || !aligned(counts, 4)) return DO_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    if (dol::signatures_fast_supported(logits, p)) {
-        cudaError_t e = cudaMemsetAsync(counts, 0, sizeof(int) * (size_t)p.L * p.E, s);
-        const dol::ZeroSpans none = {{nullptr, nullptr, nullptr}, {0, 0, 0}};
-        if (e == cudaSuccess)
-            e = dol::launch_signatures_fast(logits, p, bits, counts, nullptr, nullptr, none, nullptr,
-                                            s);
-        return from_cuda(e);
-    }
     return from_cuda(dol::launch_signatures(logits, p, bits, counts, s));
 }
 
@@ -183,25 +170,37 @@ do_status do_loss_fwd_bwd(const float *logits, const uint32_t *bits, const int32
     if (!aligned(logits, 4) || !aligned(bits, 4) || !aligned(D, 4) || !aligned(loss, 4) ||
         (dlogits && !aligned(dlogits, 4)) || (origin_do && !aligned(origin_do, 8)))
         return DO_ERR_INVALID_ARG;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < dol::workspace_bytes_plain(p))
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < dol::workspace_bytes_plain(p, false))
         return DO_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
-    if (dol::loss_fast_supported(p, logits, D, dlogits) && aligned(bits, 16)) {
-        const dol::WsLayout w = dol::ws_layout(p);
-        char *ws = static_cast<char *>(workspace);
-        int *done = reinterpret_cast<int *>(ws + w.done);
-        uint8_t *idx = reinterpret_cast<uint8_t *>(ws + w.idx);
-        cudaError_t e = dol::launch_idx_from_bits(bits, p, idx, done, p.L, s);
+    const dol::WsLayout w = dol::ws_layout_for(p, workspace_bytes, true);
+    char *ws = static_cast<char *>(workspace);
+    int *done = reinterpret_cast<int *>(ws + w.done);
+    int *status = reinterpret_cast<int *>(ws);
+    double *partials = reinterpret_cast<double *>(ws + w.partials);
+    uint8_t *idx = reinterpret_cast<uint8_t *>(ws + w.idx);
+    long long *origin = reinterpret_cast<long long *>(origin_do);
+    cudaError_t e = cudaSuccess;
+    if (w.image && dol::loss_mma_supported(p, logits, dlogits) && aligned(D, 16)) {
+        // the given matrix's image of D' and origin_do, then the tensor-core kernel
+        unsigned char *bimg = reinterpret_cast<unsigned char *>(ws + w.bimg);
+        int *img_ok = reinterpret_cast<int *>(ws + w.img_ok);
+        e = dol::launch_dprime_image(D, p, bimg, img_ok, origin, done, s);
         if (e == cudaSuccess)
-            e = dol::launch_loss_fast(logits, idx, D, nullptr, nullptr, p, gate, d_scale,
-                                      grad_scale, loss, reinterpret_cast<long long *>(origin_do),
-                                      dlogits, reinterpret_cast<double *>(ws + w.partials), done,
-                                      reinterpret_cast<int *>(ws), nullptr, s);
+            e = dol::launch_loss_mma(logits, bits, bimg, nullptr, p, gate, d_scale, grad_scale, loss,
+                                     dlogits, partials, done, status, nullptr, s, nullptr, nullptr,
+                                     img_ok, D);
         return from_cuda(e);
     }
-    return from_cuda(dol::launch_loss(logits, bits, D, p, gate, d_scale, grad_scale, loss,
-                                      reinterpret_cast<long long *>(origin_do), dlogits,
-                                      workspace, s));
+    if (dol::loss_fast_supported(p, logits, D, dlogits) && aligned(bits, 16)) {
+        e = dol::launch_idx_from_bits(bits, p, idx, done, p.L, s);
+        if (e == cudaSuccess)
+            e = dol::launch_loss_fast(logits, idx, D, nullptr, nullptr, p, gate, d_scale, grad_scale,
+                                      loss, origin, dlogits, partials, done, status, nullptr, s);
+        return from_cuda(e);
+    }
+    return from_cuda(dol::launch_loss(logits, bits, D, p, gate, d_scale, grad_scale, loss, origin,
+                                      dlogits, status, partials, s));
 }
 
 }  // extern "C"
@@ -229,97 +228,84 @@ do_status forward_backward_impl(const float *logits, int64_t T, int32_t E, int32
         (origin_do && !aligned(origin_do, 8)))
         return DO_ERR_INVALID_ARG;
     if (ra && (st = check_route(p, *ra)) != DO_OK) return st;
-    const size_t need = ra ? dol::workspace_bytes(p) : dol::workspace_bytes_plain(p);
+    const size_t need = ra ? dol::workspace_bytes(p, false) : dol::workspace_bytes_plain(p, false);
     if (!workspace || !aligned(workspace, 256) || workspace_bytes < need) return DO_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
+    const dol::WsLayout w = dol::ws_layout_for(p, workspace_bytes, !ra);
+    char *ws = static_cast<char *>(workspace);
+    int *done = reinterpret_cast<int *>(ws + w.done);
+    int *status = reinterpret_cast<int *>(ws);
+    int *rscratch = reinterpret_cast<int *>(ws + w.route_base);
+    double *partials = reinterpret_cast<double *>(ws + w.partials);
+    long long *origin = reinterpret_cast<long long *>(origin_do);
     const dol::RouteOut route = {ra ? ra->ids : nullptr, ra ? ra->combine : nullptr, gate};
-    const bool fast = dol::signatures_fast_supported(logits, p) &&
-                      dol::loss_fast_supported(p, logits, D, dlogits) && aligned(bits, 16) &&
-                      route_fast_ok(ra);
+    const bool select = dol::select_supported(logits, p);
+    // the loss kernels that take the chosen experts from the selection kernel
+    const bool loss_idx = select && aligned(bits, 16) &&
+                          (dol::loss_fast_supported(p, logits, D, dlogits) ||
+                           dol::loss_fast256_supported(p, logits, D, dlogits));
+    const bool mma = select && w.image && dol::loss_mma_supported(p, logits, dlogits);
+    uint8_t *idx = loss_idx && !mma ? reinterpret_cast<uint8_t *>(ws + w.idx) : nullptr;
     // the router GEMM runs only in the fused fast path, without routing outputs
-    if (rin && !(fast && !ra && dol::router_supported(p, rin->H, rin->X, rin->Wr, logits)))
+    if (rin && !(loss_idx && w.cooc && !ra &&
+                 dol::router_supported(p, rin->H, rin->X, rin->Wr, logits)))
         return DO_ERR_UNSUPPORTED;
-    if (fast) {
-        // signatures (+ per-CTA co-occurrence counts) -> reduction to C -> loss,
-        // which builds D = n_i + n_j - 2 c_ij and writes D and the counts
-        const dol::WsLayout w = dol::ws_layout(p);
-        char *ws = static_cast<char *>(workspace);
-        int *done = reinterpret_cast<int *>(ws + w.done);
-        uint8_t *idx = reinterpret_cast<uint8_t *>(ws + w.idx);
+    cudaError_t e;
+    int *n_acc = nullptr;
+    if (select && w.cooc) {
+        // signatures + per-CTA co-occurrence counts -> reduction, which builds
+        // D = n_i + n_j - 2 c_ij and writes D, the counts and origin_do
         uint32_t *parts = reinterpret_cast<uint32_t *>(ws + w.cooc_parts);
-        int *n_acc = reinterpret_cast<int *>(ws + w.n_acc);
+        n_acc = reinterpret_cast<int *>(ws + w.n_acc);
         // origin_do is summed by the reduction kernel (integer atomics) and
         // status_out ORed by the loss kernel: zero them first
         const dol::ZeroSpans zero = {{done, reinterpret_cast<int *>(origin_do), status_out},
                                      {(int64_t)p.L, origin_do ? 2 * (int64_t)p.L : 0,
                                       status_out ? 1 : 0}};
-        int *status = reinterpret_cast<int *>(ws);
-        // D <= T here (one window of tokens): the two-piece fp16 split of the
-        // tensor-core path is exact when R < 2^23 (checked by loss_mma_supported)
-        const bool mma = dol::loss_mma_supported(p, gate, logits, D, dlogits);
+        const bool big = dol::loss_mma_big(p);
         unsigned char *bimg = mma ? reinterpret_cast<unsigned char *>(ws + w.bimg) : nullptr;
-        cudaError_t e =
-            rin ? dol::launch_router_signatures(rin->X, rin->Wr, rin->H, const_cast<float *>(logits),
+        const dol::SelectOut so = {bits, n_acc, idx, parts, zero, status, route};
+        e = rin ? dol::launch_router_signatures(rin->X, rin->Wr, rin->H, const_cast<float *>(logits),
                                                 p, bits, n_acc, idx, parts, zero, status, s)
-            : ra ? dol::launch_signatures_fast_routed(logits, p, bits, n_acc, idx, parts, zero,
-                                                      status, route, s)
-                 : dol::launch_signatures_fast(logits, p, bits, n_acc, idx, parts, zero, status, s);
-        const int P1 = rin ? dol::router_ctas_per_problem(p) : dol::sig_fast_ctas_per_problem(p);
-        int *rscratch = reinterpret_cast<int *>(ws + w.route_base);
+                : dol::launch_select(logits, p, so, s);
+        const int P1 = rin ? dol::router_ctas_per_problem(p) : dol::sig_ctas_per_problem(p);
         if (e == cudaSuccess)
-            e = dol::launch_cooc_reduce(parts, P1, n_acc, p, D, counts, bimg,
-                                        reinterpret_cast<long long *>(origin_do), s);
-        if (e == cudaSuccess) {
-            if (mma)
-                e = dol::launch_loss_mma(logits, idx, bimg, n_acc, p, 1.0f, grad_scale, loss, dlogits,
-                                         reinterpret_cast<double *>(ws + w.partials), done, status,
-                                         status_out, s);
-            else
-                e = dol::launch_loss_fast(logits, idx, D, counts, n_acc, p, gate, 1.0f, grad_scale,
-                                          loss, nullptr, dlogits,
-                                          reinterpret_cast<double *>(ws + w.partials), done,
-                                          status, status_out, s);
+            e = dol::launch_cooc_reduce(parts, P1, n_acc, p, D, counts, bimg, big, origin, s);
+        if (e == cudaSuccess && mma) {
+            e = dol::launch_loss_mma(logits, bits, bimg, n_acc, p, gate, 1.0f, grad_scale, loss, dlogits,
+                                     partials, done, status, status_out, s);
+            if (e == cudaSuccess && status_done) *status_done = status_out != nullptr;
+            if (e == cudaSuccess && ra)
+                e = dol::launch_route_dispatch(bits, ra->ids, p, ra->offsets, ra->rows, ra->pos,
+                                               rscratch, s);
+            return from_cuda(e);
         }
-        // the dispatch order (from the signatures and ids alone) follows the loss kernel
-        if (e == cudaSuccess && ra)
-            e = dol::launch_route_dispatch(bits, ra->ids, p, ra->offsets, ra->rows, ra->pos,
-                                           rscratch, s);
-        if (e == cudaSuccess && status_done) *status_done = status_out != nullptr;
-        return from_cuda(e);
-    }
-    if (!ra && dol::signatures_fast256_supported(logits, p) && aligned(bits, 16) &&
-        dol::loss_fast256_supported(p, logits, D, dlogits)) {
-        // E = 256: the fast selection (with the chosen experts), the Hamming
-        // matrix from the signatures, and the ALU loss kernel with D in
-        // shared-memory planes
-        const dol::WsLayout w = dol::ws_layout(p);
-        char *ws = static_cast<char *>(workspace);
-        int *done = reinterpret_cast<int *>(ws + w.done);
-        uint8_t *idx = reinterpret_cast<uint8_t *>(ws + w.idx);
-        int *status = reinterpret_cast<int *>(ws);
+        origin = nullptr;  // written
+    } else {
+        // the Hamming matrix from the signatures
         const dol::ZeroSpans zero = {{done, status_out, nullptr},
                                      {(int64_t)p.L, status_out ? 1 : 0, 0}};
-        cudaError_t e = cudaMemsetAsync(counts, 0, sizeof(int) * (size_t)p.L * p.E, s);
-        if (e == cudaSuccess)
-            e = dol::launch_signatures_fast256(logits, p, bits, counts, idx, zero, status, s);
+        e = cudaMemsetAsync(counts, 0, sizeof(int) * (size_t)p.L * p.E, s);
+        if (e == cudaSuccess) {
+            const dol::SelectOut so = {bits, counts, idx, nullptr, zero, status, route};
+            e = select ? dol::launch_select(logits, p, so, s)
+                       : dol::launch_signatures(logits, p, bits, counts, s, route);
+        }
         if (e == cudaSuccess) e = dol::launch_hamming(bits, p, D, s);
-        if (e == cudaSuccess)
-            e = dol::launch_loss_fast(logits, idx, D, counts, nullptr, p, gate, 1.0f, grad_scale,
-                                      loss, reinterpret_cast<long long *>(origin_do), dlogits,
-                                      reinterpret_cast<double *>(ws + w.partials), done, status,
-                                      status_out, s);
-        if (e == cudaSuccess && status_done) *status_done = status_out != nullptr;
-        return from_cuda(e);
     }
-    cudaError_t e = dol::launch_signatures(logits, p, bits, counts, s, route);
-    if (e == cudaSuccess) e = dol::launch_hamming(bits, p, D, s);
-    if (e == cudaSuccess)
-        e = dol::launch_loss(logits, bits, D, p, gate, 1.0f, grad_scale, loss,
-                             reinterpret_cast<long long *>(origin_do), dlogits, workspace, s);
+    if (e == cudaSuccess) {
+        if (loss_idx) {
+            e = dol::launch_loss_fast(logits, idx, D, counts, n_acc, p, gate, 1.0f, grad_scale,
+                                      loss, origin, dlogits, partials, done, status, status_out, s);
+            if (e == cudaSuccess && status_done) *status_done = status_out != nullptr;
+        } else {
+            e = dol::launch_loss(logits, bits, D, p, gate, 1.0f, grad_scale, loss, origin, dlogits,
+                                 status, partials, s, n_acc);
+        }
+    }
+    // the dispatch order (from the signatures and ids alone) follows the loss kernel
     if (e == cudaSuccess && ra)
-        e = dol::launch_route_dispatch(
-            bits, ra->ids, p, ra->offsets, ra->rows, ra->pos,
-            reinterpret_cast<int *>(static_cast<char *>(workspace) + dol::ws_layout(p).route_base), s);
+        e = dol::launch_route_dispatch(bits, ra->ids, p, ra->offsets, ra->rows, ra->pos, rscratch, s);
     return from_cuda(e);
 }
 
@@ -371,14 +357,14 @@ do_status do_router_forward_backward(const void *X, const void *Wr, int64_t T, i
 // the choice depends only on the logits, bits and D pointers and the shape,
 // which both halves receive.
 bool split_fast(const Problem &p, const float *logits, const uint32_t *bits, const int *D) {
-    return dol::signatures_fast_supported(logits, p) &&
+    return dol::select_supported(logits, p) &&
            dol::loss_fast_supported(p, logits, D, nullptr) && aligned(bits, 16);
 }
 
 // Whether the forward half writes the fp16 image of D' for the tensor-core
-// loss kernel (dlogits is not known there: the logits' alignment stands in).
-bool split_mma(const Problem &p, int gate, const float *logits, const int *D) {
-    return dol::loss_mma_supported(p, gate, logits, D, logits);
+// loss kernel (dlogits is not known there).
+bool split_mma(const Problem &p, const float *logits, const dol::WsLayout &w) {
+    return dol::select_supported(logits, p) && w.image && dol::loss_mma_supported(p, logits, nullptr);
 }
 
 do_status do_routed_forward(const float *logits, int64_t T, int32_t E, int32_t k, int32_t L,
@@ -401,51 +387,41 @@ do_status do_routed_forward(const float *logits, int64_t T, int32_t E, int32_t k
     const RouteArgs ra = {expert_ids, combine, expert_offsets, dispatch_rows, dispatch_pos};
     if (routed && (st = check_route(p, ra)) != DO_OK) return st;
     if (!routed && (expert_offsets || dispatch_rows || dispatch_pos)) return DO_ERR_INVALID_ARG;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < dol::workspace_bytes(p))
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < dol::workspace_bytes(p, false))
         return DO_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
     char *ws = static_cast<char *>(workspace);
-    const dol::WsLayout w = dol::ws_layout(p);
+    const dol::WsLayout w = dol::ws_layout_for(p, workspace_bytes, false);
     int *rscratch = reinterpret_cast<int *>(ws + w.route_base);
     const dol::RouteOut route = {expert_ids, combine, gate};
-    const RouteArgs *rap = routed ? &ra : nullptr;
     cudaError_t e = cudaSuccess;
-    if (split_fast(p, logits, bits, D)) {
+    int *n_acc = nullptr;
+    if (dol::select_supported(logits, p) && w.cooc) {
         int *done = reinterpret_cast<int *>(ws + w.done);
-        uint8_t *idx = reinterpret_cast<uint8_t *>(ws + w.idx);
         uint32_t *parts = reinterpret_cast<uint32_t *>(ws + w.cooc_parts);
-        int *n_acc = reinterpret_cast<int *>(ws + w.n_acc);
-        int *status = reinterpret_cast<int *>(ws);
+        n_acc = reinterpret_cast<int *>(ws + w.n_acc);
         const dol::ZeroSpans zero = {{done, reinterpret_cast<int *>(origin_do), nullptr},
                                      {(int64_t)p.L, origin_do ? 2 * (int64_t)p.L : 0, 0}};
-        unsigned char *bimg =
-            split_mma(p, gate, logits, D) ? reinterpret_cast<unsigned char *>(ws + w.bimg) : nullptr;
-        if (routed && !route_fast_ok(rap))  // unaligned routing outputs: the generic selection
-            e = dol::launch_signatures(logits, p, bits, counts, s, route);
+        // what the backward half's loss kernel reads
+        unsigned char *bimg = split_mma(p, logits, w)
+                                  ? reinterpret_cast<unsigned char *>(ws + w.bimg) : nullptr;
+        const dol::SelectOut so = {bits, n_acc, nullptr, parts, zero, reinterpret_cast<int *>(ws), route};
+        e = dol::launch_select(logits, p, so, s);
         if (e == cudaSuccess)
-            e = routed && route_fast_ok(rap)
-                    ? dol::launch_signatures_fast_routed(logits, p, bits, n_acc, idx, parts, zero,
-                                                         status, route, s)
-                    : dol::launch_signatures_fast(logits, p, bits, n_acc, idx, parts, zero, status, s);
-        if (e == cudaSuccess)
-            e = dol::launch_cooc_reduce(parts, dol::sig_fast_ctas_per_problem(p), n_acc, p, D,
-                                        counts, bimg, reinterpret_cast<long long *>(origin_do), s);
-        // no loss kernel follows in this call: the dispatch kernels clear the
-        // counts accumulator
-        if (e == cudaSuccess)
-            e = dol::launch_route_dispatch(bits, expert_ids, p, expert_offsets, dispatch_rows,
-                                           dispatch_pos, rscratch, s, n_acc);
-        return from_cuda(e);
+            e = dol::launch_cooc_reduce(parts, dol::sig_ctas_per_problem(p), n_acc, p, D,
+                                        counts, bimg, dol::loss_mma_big(p),
+                                        reinterpret_cast<long long *>(origin_do), s);
     } else {
-        e = routed ? dol::launch_signatures(logits, p, bits, counts, s, route)
-                   : dol::launch_signatures(logits, p, bits, counts, s);
+        e = dol::launch_signatures(logits, p, bits, counts, s, route);
         if (e == cudaSuccess) e = dol::launch_hamming(bits, p, D, s);
         if (e == cudaSuccess && origin_do)
             e = dol::launch_origin_do(D, p, reinterpret_cast<long long *>(origin_do), s);
     }
+    // no loss kernel follows in this call: the dispatch kernels clear the
+    // counts accumulator
     if (e == cudaSuccess)
         e = dol::launch_route_dispatch(bits, expert_ids, p, expert_offsets, dispatch_rows,
-                                       dispatch_pos, rscratch, s);
+                                       dispatch_pos, rscratch, s, n_acc);
     return from_cuda(e);
 }
 
@@ -468,11 +444,11 @@ do_status do_routed_backward(const float *logits, int64_t T, int32_t E, int32_t 
         (rg && (!aligned(expert_ids, 4) || !aligned(grad_combine, 4))) || !aligned(loss, 4) ||
         !aligned(dlogits, 4))
         return DO_ERR_INVALID_ARG;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < dol::workspace_bytes(p))
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < dol::workspace_bytes(p, false))
         return DO_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
     char *ws = static_cast<char *>(workspace);
-    const dol::WsLayout w = dol::ws_layout(p);
+    const dol::WsLayout w = dol::ws_layout_for(p, workspace_bytes, false);
     int *status = reinterpret_cast<int *>(ws);
     int *done = reinterpret_cast<int *>(ws + w.done);
     uint8_t *idx = reinterpret_cast<uint8_t *>(ws + w.idx);
@@ -482,47 +458,32 @@ do_status do_routed_backward(const float *logits, int64_t T, int32_t E, int32_t 
     // forward half left for the tensor-core kernel; otherwise D is a matrix
     // summed over ranks or micro-batches (Eq. global_do), read as given.
     const bool local = d_scale == 1.0f;
+    const bool mma = split_mma(p, logits, w) && dol::loss_mma_supported(p, logits, dlogits);
+    unsigned char *bimg = reinterpret_cast<unsigned char *>(ws + w.bimg);
     cudaError_t e;
-    if (!local && split_fast(p, logits, bits, D) && aligned(dlogits, 16) &&
-        dol::loss_mma_supported(p, gate, logits, D, dlogits, true) &&
-        (!rg || (aligned(expert_ids, 16) && aligned(grad_combine, 16)))) {
-        // a given matrix: its image of D' is built here, with a flag per
-        // problem saying whether the two fp16 pieces hold it exactly; the
-        // tensor-core kernel takes the exact problems (routing gradient in its
-        // epilogue), the ALU kernel and the routing-gradient kernel the others
-        unsigned char *bimg = reinterpret_cast<unsigned char *>(ws + w.bimg);
-        int *img_ok = reinterpret_cast<int *>(ws + w.img_ok);
-        e = dol::launch_dprime_image(D, p, bimg, img_ok, s);
+    if (mma && (local || aligned(D, 16))) {
+        // a given matrix: its image of D' is built here
+        int *img_ok = local ? nullptr : reinterpret_cast<int *>(ws + w.img_ok);
+        e = local ? cudaSuccess : dol::launch_dprime_image(D, p, bimg, img_ok, nullptr, nullptr, s);
+        // the routing gradient is added in the loss kernel's epilogue where it
+        // can, else by its own kernel
+        const bool rg_mma = rg && dol::loss_mma_route_grad(p, gate, expert_ids, grad_combine);
         if (e == cudaSuccess)
-            e = dol::launch_loss_mma(logits, idx, bimg, nullptr, p, d_scale, grad_scale, loss,
-                                     dlogits, partials, done, status, nullptr, s, expert_ids,
-                                     grad_combine, img_ok);
-        if (e == cudaSuccess)
-            e = dol::launch_loss_fast(logits, idx, D, nullptr, nullptr, p, gate, d_scale,
-                                      grad_scale, loss, nullptr, dlogits, partials, done, status,
-                                      nullptr, s, img_ok);
-        if (e == cudaSuccess && rg)
-            e = dol::launch_route_backward(logits, expert_ids, grad_combine, p.T * p.L, E, k, gate,
-                                           1, dlogits, status, s, img_ok, p.T);
-        return from_cuda(e);
-    }
-    if (split_fast(p, logits, bits, D) && aligned(dlogits, 16)) {
-        if (local && split_mma(p, gate, logits, D) &&
-            dol::loss_mma_supported(p, gate, logits, D, dlogits) &&
-            (!rg || (aligned(expert_ids, 16) && aligned(grad_combine, 16)))) {
-            // the routing gradient is added in the loss kernel's epilogue
-            return from_cuda(dol::launch_loss_mma(
-                logits, idx, reinterpret_cast<unsigned char *>(ws + w.bimg), n_acc, p, 1.0f,
-                grad_scale, loss, dlogits, partials, done, status, nullptr, s, expert_ids,
-                grad_combine));
-        }
+            e = dol::launch_loss_mma(logits, bits, bimg, local ? n_acc : nullptr, p, gate, d_scale,
+                                     grad_scale, loss, dlogits, partials, done, status, nullptr, s,
+                                     rg_mma ? expert_ids : nullptr, rg_mma ? grad_combine : nullptr,
+                                     img_ok, local ? nullptr : D);
+        if (rg_mma) return from_cuda(e);
+    } else if (split_fast(p, logits, bits, D) && aligned(dlogits, 16)) {
+        e = dol::launch_idx_from_bits(bits, p, idx, nullptr, 0, s);
         // the row sums of D come from the counts only for the local matrix
-        e = dol::launch_loss_fast(logits, idx, D, local ? counts : nullptr, n_acc, p, gate,
-                                  d_scale, grad_scale, loss, nullptr, dlogits, partials, done,
-                                  status, nullptr, s);
+        if (e == cudaSuccess)
+            e = dol::launch_loss_fast(logits, idx, D, local ? counts : nullptr, n_acc, p, gate,
+                                      d_scale, grad_scale, loss, nullptr, dlogits, partials, done,
+                                      status, nullptr, s);
     } else {
         e = dol::launch_loss(logits, bits, D, p, gate, d_scale, grad_scale, loss, nullptr, dlogits,
-                             workspace, s);
+                             status, partials, s);
     }
     // elsewhere the routing gradient is added by its own kernel
     if (e == cudaSuccess && rg)
@@ -551,12 +512,13 @@ do_status do_routing(const float *logits, int64_t T, int32_t E, int32_t k, int32
     const dol::RouteOut route = {expert_ids, combine, gate};
     cudaError_t e;
     int *rscratch = reinterpret_cast<int *>(ws + dol::kWsHeader + routing_bits_bytes(p));
-    if (dol::signatures_fast_supported(logits, p) && route_fast_ok(&ra)) {
+    if (dol::select_supported(logits, p)) {
         // the selection kernel writes no counts: the dispatch scan takes them
         // from the signatures' popcounts (no memset between the kernels)
         const dol::ZeroSpans none = {{nullptr, nullptr, nullptr}, {0, 0, 0}};
-        e = dol::launch_signatures_fast_routed(logits, p, bits, nullptr, nullptr, nullptr, none,
-                                               reinterpret_cast<int *>(ws), route, s);
+        const dol::SelectOut so = {bits, nullptr, nullptr, nullptr, none, reinterpret_cast<int *>(ws),
+                                   route};
+        e = dol::launch_select(logits, p, so, s);
         if (e == cudaSuccess)
             e = dol::launch_route_dispatch(bits, expert_ids, p, expert_offsets, dispatch_rows,
                                            dispatch_pos, rscratch, s, nullptr, counts);

@@ -70,20 +70,33 @@ struct ZeroSpans {
 //   cooc_parts      [L][P1][triangle words] uint32, per-CTA co-occurrence counts
 //   n_acc           [L][E] int32, counts summed by the signatures CTAs (kept at
 //                   zero between calls: the loss kernel clears it after use)
-//   bimg            [L][kBImageBytes], the fp16 image of D' (E = 128 only)
+//   bimg            [L][bimg_bytes(EP)], the fp16 image of D' (E <= 128)
 //   img_ok          [L] int32, 1 where the image of a given (summed) D is exact
 //   route_base      route_scratch_ints int32, scratch of the dispatch order
 struct WsLayout {
     size_t done, partials, idx, cooc_parts, n_acc, bimg, img_ok, route_base, total;
     int max_parts;  // partial slots per problem
+    bool cooc;      // the layout has cooc_parts and n_acc
+    bool image;     // ... and bimg
 };
 // Signatures CTAs per problem on the fast path: min(SMs, kMaxSigCtas) / L.
-constexpr int kMaxSigCtas = 256;
+constexpr int kMaxSigCtas = 255;
 int max_sig_ctas_per_problem(const Problem &p);
-WsLayout ws_layout(const Problem &p);
-inline size_t workspace_bytes(const Problem &p) { return ws_layout(p).total; }
+// wide: with room for the co-occurrence triangles at every size that has them
+// (cooc_sizes_ok); without it only E in {32, 64, 128}, k in {1, 2, 4, 8} have
+// it and the other sizes take D from the signatures (a fixed scratch array
+// that is too small for the triangles still serves them).
+WsLayout ws_layout(const Problem &p, bool wide);
+inline size_t workspace_bytes(const Problem &p, bool wide = true) { return ws_layout(p, wide).total; }
 // What a call without routing outputs needs: the layout up to the routing scratch.
-inline size_t workspace_bytes_plain(const Problem &p) { return ws_layout(p).route_base; }
+inline size_t workspace_bytes_plain(const Problem &p, bool wide = true) {
+    return ws_layout(p, wide).route_base;
+}
+// The layout a call of `bytes` workspace uses.
+inline WsLayout ws_layout_for(const Problem &p, size_t bytes, bool plain) {
+    const WsLayout w = ws_layout(p, true);
+    return (plain ? w.route_base : w.total) <= bytes ? w : ws_layout(p, false);
+}
 
 // Number of generic loss-kernel CTAs per problem; fixes the partial-sum
 // layout and therefore the reduction order.
@@ -95,14 +108,35 @@ cudaError_t launch_signatures(const float *logits, const Problem &p, uint32_t *b
                               int *counts, cudaStream_t s,
                               const RouteOut &route = RouteOut{nullptr, nullptr, 0});
 cudaError_t launch_hamming(const uint32_t *bits, const Problem &p, int *D, cudaStream_t s);
-// The fast selection at E = 256 (k in {1, 2, 4, 8}, 16-byte aligned logits):
-// signatures and counts (counts zero on entry), no co-occurrence; idx (may be
-// null) the chosen experts of every token; zero: ranges cleared for the
-// kernels after it; status (may be null): the device status word.
-bool signatures_fast256_supported(const float *logits, const Problem &p);
-cudaError_t launch_signatures_fast256(const float *logits, const Problem &p, uint32_t *bits,
-                                      int *counts, uint8_t *idx, const ZeroSpans &zero,
-                                      int *status, cudaStream_t s);
+// The selection kernel of select.cuh (E <= 512 a multiple of 4, k <= 16,
+// 16-byte aligned logits).  counts: zero on entry; null: not counted.  idx
+// (may be null, E <= 256): the chosen experts of every token, one byte each.
+// zero: ranges cleared for the kernels after it.  status (may be null): the
+// device status word.  cooc (E <= 256, may be null): the per-CTA co-occurrence
+// triangles, sig_ctas_per_problem of them per problem; counts is then the
+// accumulator that the reduction reads.
+struct SelectOut {
+    uint32_t *bits;
+    int *counts;
+    uint8_t *idx;
+    uint32_t *cooc;
+    ZeroSpans zero;
+    int *status;
+    RouteOut route;
+};
+// sig_fast.cuh's kernel at the sizes of signatures_fast_supported (with routing
+// outputs, ids and combine 16-byte aligned), else the one of select.cuh.
+bool signatures_fast_supported(const float *logits, const Problem &p);
+cudaError_t launch_signatures_fast(const float *logits, const Problem &p, uint32_t *bits,
+                                   int *counts, uint8_t *idx, uint32_t *cooc, const ZeroSpans &zero,
+                                   int *status, cudaStream_t s);
+cudaError_t launch_signatures_fast_routed(const float *logits, const Problem &p, uint32_t *bits,
+                                          int *counts, uint8_t *idx, uint32_t *cooc,
+                                          const ZeroSpans &zero, int *status,
+                                          const RouteOut &route, cudaStream_t s);
+bool select_supported(const float *logits, const Problem &p);
+cudaError_t launch_select(const float *logits, const Problem &p, const SelectOut &o, cudaStream_t s);
+int sig_ctas_per_problem(const Problem &p);
 cudaError_t launch_add_distances(const int *D, int *D_sum, int64_t n, cudaStream_t s);
 cudaError_t launch_hamming_accumulate(const uint32_t *bits, const Problem &p, int *D, cudaStream_t s);
 cudaError_t launch_origin_do(const int *D, const Problem &p, long long *origin_do, cudaStream_t s);
@@ -110,21 +144,12 @@ cudaError_t launch_origin_do(const int *D, const Problem &p, long long *origin_d
 // local Hamming matrix from its origin_do (App. C.1).
 cudaError_t launch_offdiag_variance(const long long *origin_do, const Problem &p, double *var,
                                     cudaStream_t s);
+// Generic loss (any E, k): n_zero ([L][E], may be null) is cleared.
 cudaError_t launch_loss(const float *logits, const uint32_t *bits, const int *D,
                         const Problem &p, int gate, float d_scale, float grad_scale,
-                        float *loss, long long *origin_do, float *dlogits, void *workspace,
-                        cudaStream_t s);
+                        float *loss, long long *origin_do, float *dlogits, int *status,
+                        double *partials, cudaStream_t s, int *n_zero = nullptr);
 
-// Fast paths (E in {32, 64, 128}, k in {1, 2, 4, 8}, 16-byte aligned rows).
-bool signatures_fast_supported(const float *logits, const Problem &p);
-cudaError_t launch_signatures_fast(const float *logits, const Problem &p, uint32_t *bits,
-                                   int *counts, uint8_t *idx, uint32_t *cooc, const ZeroSpans &zero,
-                                   int *status, cudaStream_t s);
-// The same kernel with the routing outputs (ids and combine 16-byte aligned).
-cudaError_t launch_signatures_fast_routed(const float *logits, const Problem &p, uint32_t *bits,
-                                          int *counts, uint8_t *idx, uint32_t *cooc,
-                                          const ZeroSpans &zero, int *status,
-                                          const RouteOut &route, cudaStream_t s);
 // Dispatch order of the routed (token, choice) pairs from the signatures and
 // the chosen ids alone: offsets [L][E+1], rows [L][T k], pos [L][T][k] (each
 // may be null).  scratch: route_scratch_ints(p) ints.  Launched as
@@ -132,13 +157,10 @@ cudaError_t launch_signatures_fast_routed(const float *logits, const Problem &p,
 int64_t route_chunks(const Problem &p);
 int64_t route_scratch_ints(const Problem &p);
 // Backward of the combine weights to the logits over `rows` token rows
-// (route_bwd.cu); status bit 2 for an id outside [0, E).  skip (with
-// accumulate only; may be null): [rows / layer_rows] flags, the rows of a
-// problem whose flag is nonzero are left alone.
+// (route_bwd.cu); status bit 2 for an id outside [0, E).
 cudaError_t launch_route_backward(const float *z, const int32_t *ids, const float *g, int64_t rows,
                                   int32_t E, int32_t k, int32_t gate, int32_t accumulate,
-                                  float *dz, int32_t *status_flags, cudaStream_t s,
-                                  const int *skip = nullptr, int64_t layer_rows = 0);
+                                  float *dz, int32_t *status_flags, cudaStream_t s);
 
 // n_zero (may be null): an [L][E] accumulator cleared once the kernels before
 // these have finished (the scan kernel does it after its dependency wait).
@@ -166,39 +188,46 @@ cudaError_t launch_idx_from_bits(const uint32_t *bits, const Problem &p, uint8_t
 // counts: when given, R_i = (E - 2k) n_i + T k (D local to these tokens) and
 // n_zero ([L][E], may be null) is cleared once D is read; otherwise R_i is a
 // column sum of D.
-// Tensor-core loss path (E = 128, sigmoid-norm gate, k in {1,2,4,8}, T <= 2^22).
-bool loss_mma_supported(const Problem &p, int gate, const float *logits, const int *D,
-                        const float *dlogits, bool image_checked = false);
-int loss_mma_ctas_per_problem(const Problem &p);
-// bimg: the fp16 image of D' written by launch_cooc_reduce for these tokens
-// (which also gives origin_do on this path).
-cudaError_t launch_loss_mma(const float *logits, const uint8_t *idx, const unsigned char *bimg,
-                            int *n_zero, const Problem &p, float d_scale, float grad_scale,
+// Tensor-core loss path (loss_mma.cuh).  bimg: the image of D' written by
+// launch_cooc_reduce for these tokens (marker diagonal where loss_mma_big), or
+// by launch_dprime_image for a given matrix D (where img_ok is 0, D is read
+// instead).  dlogits may be
+// null (forward only).
+bool loss_mma_supported(const Problem &p, const float *logits, const float *dlogits);
+bool loss_mma_big(const Problem &p);
+bool loss_mma_route_grad(const Problem &p, int gate, const int *ids, const float *g);
+cudaError_t launch_loss_mma(const float *logits, const uint32_t *bits, const unsigned char *bimg,
+                            int *n_zero, const Problem &p, int gate, float d_scale, float grad_scale,
                             float *loss, float *dlogits, double *partials, int *done, int *status,
                             int *status_out, cudaStream_t s, const int *rg_ids = nullptr,
-                            const float *rg_g = nullptr, const int *img_ok = nullptr);
+                            const float *rg_g = nullptr, const int *img_ok = nullptr,
+                            const int *D = nullptr);
 cudaError_t launch_loss_fast(const float *logits, const uint8_t *idx, const int *D,
                              const int *counts, int *n_zero, const Problem &p, int gate,
                              float d_scale, float grad_scale, float *loss, long long *origin_do,
                              float *dlogits, double *partials, int *done, int *status,
-                             int *status_out, cudaStream_t s, const int *img_ok = nullptr);
+                             int *status_out, cudaStream_t s);
 
-// Co-occurrence counts c_ab (a <= b) of one CTA are kept as a triangle whose
-// row a holds columns (a & ~3) .. E-1, so that every row starts 16-byte
-// aligned.  Offset of row a: sum over a' < a of (E - 4 floor(a'/4)).
-template <int E>
-__host__ __device__ constexpr int cooc_row_offset(int a) {
-    return a * E - 8 * (a / 4) * (a / 4 - 1) - 4 * (a % 4) * (a / 4);
-}
+// Co-occurrence counts c_ab (a <= b) of one CTA are kept as a triangle in
+// chunks of four columns: chunk c = b / 4 holds rows 0 .. 4c + 3, four words
+// each, so that the rows of a chunk are consecutive (a warp that holds a row
+// per lane stores 512 contiguous bytes).  Word of (a, b): tri_chunk(b / 4) +
+// 4 a + b % 4.  n, the width, is E rounded up to 32 (cooc_width).
+__host__ __device__ constexpr int tri_chunk(int c) { return 8 * c * (c + 1); }
+__host__ __device__ constexpr int tri_words(int n) { return tri_chunk(n / 4); }
 
-// The matrix D' of the tensor-core loss kernel (E = 128): D'_ab = D_ab off the
+// The matrix D' of the tensor-core loss kernel (E <= 128): D'_ab = D_ab off the
 // diagonal, D'_aa = -R_a, stored as two fp16 pieces D' = 2048 hi + lo, both
-// exact: off the diagonal (0 <= D <= 2^16) hi = D >> 11 and lo = D & 2047; on
+// exact: off the diagonal (0 <= D < 2^22) hi = D >> 11 and lo = D & 2047; on
 // the diagonal (0 <= R < 2^23) -R = 2048 (-a) + (-b) with a = 2 round(R / 4096)
-// even and |b| <= 2048.  The image is the shared-memory operand B of that
-// kernel: rows n = 0..127 hold hi of column n, rows 128 + n lo, K-major with
-// 128-byte swizzle (two K atoms of 64 columns, 256 rows of 128 bytes each).
-constexpr int kBImageBytes = 2 * 256 * 128;
+// even and |b| <= 2048, or the marker hi = -32768, lo = 0.  The stored values
+// are half of the pieces (the selections F hold 2 instead of 1).  The image is
+// the shared-memory operand B of that kernel for EP = E rounded up to 32: rows
+// n = 0..EP-1 hold hi of column n, rows EP + n lo, K-major with 128-byte swizzle
+// (K atoms of 64 columns, 2 EP rows of 128 bytes each), then R as EP fp32.
+inline bool bimg_sizes_ok(int E, int k) { return E % 4 == 0 && E <= 128 && k <= 16; }
+__host__ __device__ constexpr int bimg_r_offset(int EP) { return (EP + 63) / 64 * 2 * EP * 128; }
+__host__ __device__ constexpr int bimg_bytes(int EP) { return bimg_r_offset(EP) + 4 * EP; }
 __host__ __device__ __forceinline__ uint32_t sw128_k16_offset(int row, int k, int rows) {
     const int atom = k >> 6, kc = k & 63;
     return (uint32_t)(atom * rows * 128 + row * 128 + ((((kc >> 3) ^ (row & 7))) << 4) + (kc & 7) * 2);
@@ -214,27 +243,37 @@ __host__ __device__ __forceinline__ void dprime_pieces(bool diag, int v, int *hi
     }
 }
 
-// Writes the two fp16 pieces of D'_{n,k} (dprime_pieces) into the image at
-// row n (hi) and row 128 + n (lo), column k.
-__device__ __forceinline__ void put_dprime(unsigned char *img, int n, int k, bool diag, int v) {
+__device__ __forceinline__ __half half_piece(int v) { return __float2half_rn(0.5f * (float)v); }
+
+// Writes the two fp16 pieces of D'_{n,k} into the image of EP experts at row n
+// (hi) and row EP + n (lo), column k.
+__device__ __forceinline__ void put_pieces(unsigned char *img, int EP, int n, int k, int h, int l) {
+    *reinterpret_cast<__half *>(img + sw128_k16_offset(n, k, 2 * EP)) = half_piece(h);
+    *reinterpret_cast<__half *>(img + sw128_k16_offset(EP + n, k, 2 * EP)) = half_piece(l);
+}
+__device__ __forceinline__ void put_dprime(unsigned char *img, int EP, int n, int k, bool diag, int v) {
     int h, l;
     dprime_pieces(diag, v, &h, &l);
-    *reinterpret_cast<__half *>(img + sw128_k16_offset(n, k, 256)) = __int2half_rn(h);
-    *reinterpret_cast<__half *>(img + sw128_k16_offset(128 + n, k, 256)) = __int2half_rn(l);
+    put_pieces(img, EP, n, k, h, l);
 }
 
-int sig_fast_ctas_per_problem(const Problem &p);
-size_t cooc_partial_words(int E);
-// bimg ([L][kBImageBytes], E = 128 only, may be null): the fp16 image of D'
-// for the tensor-core loss kernel, written alongside D.  origin_do (may be
+// Whether the selection kernel can leave co-occurrence counts, the width of
+// its triangles and their words.
+inline bool cooc_sizes_ok(int E, int k) { return E % 4 == 0 && E <= 256 && k <= 16; }
+inline int cooc_width(int E) { return (E + 31) / 32 * 32; }
+inline size_t cooc_partial_words(int E) { return (size_t)tri_words(cooc_width(E)); }
+// bimg ([L][bimg_bytes(EP)], E <= 128, may be null): the fp16 image of D' for
+// the tensor-core loss kernel, written alongside D (big: the marker diagonal).  origin_do (may be
 // null) must be zero on entry: sum_{a != b} D_ab^2 is added to it.
 cudaError_t launch_cooc_reduce(const uint32_t *partials, int P1, const int *n_acc, const Problem &p,
-                               int *D, int *counts, unsigned char *bimg, long long *origin_do,
-                               cudaStream_t s);
-// The image of D' from a given [L][128][128] matrix D (summed over ranks or
-// micro-batches), and img_ok [L] = 1 where its two fp16 pieces are exact.
+                               int *D, int *counts, unsigned char *bimg, bool big,
+                               long long *origin_do, cudaStream_t s);
+// The image of D' from a given [L][E][E] matrix D (16-byte aligned; the split
+// entry point's, or summed over ranks or micro-batches) with the marker
+// diagonal, img_ok [L] = 1 where it is exact, and with it Eq. origin_do and
+// cleared done counters (each may be null).
 cudaError_t launch_dprime_image(const int *D, const Problem &p, unsigned char *bimg, int *img_ok,
-                                cudaStream_t s);
+                                long long *origin_do, int *done, cudaStream_t s);
 
 // ---------------------------------------------------------------- device helpers
 

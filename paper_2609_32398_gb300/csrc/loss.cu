@@ -163,7 +163,8 @@ loss_generic_kernel(const float *__restrict__ logits, const uint32_t *__restrict
 // = sum_{i != j} D_ij^2 (Eq. origin_do), exact in int64.
 __global__ void __launch_bounds__(256)
 loss_finalize_kernel(const double *__restrict__ partials, int P, const int *__restrict__ Dg, int E,
-                     double scale, float *__restrict__ loss, long long *__restrict__ origin_do) {
+                     double scale, float *__restrict__ loss, long long *__restrict__ origin_do,
+                     int *__restrict__ n_zero) {
     __shared__ long long s_red[256];
     __shared__ double s_dred[256];
     const int layer = blockIdx.x;
@@ -171,6 +172,9 @@ loss_finalize_kernel(const double *__restrict__ partials, int P, const int *__re
         const double s = block_sum_fixed(partials + (int64_t)layer * P, P, s_dred, 256);
         if (threadIdx.x == 0) loss[layer] = (float)(s * scale);
     }
+    // the counts accumulator has been read: cleared for the next call
+    if (n_zero)
+        for (int i = threadIdx.x; i < E; i += blockDim.x) n_zero[(int64_t)layer * E + i] = 0;
     if (origin_do) {
         const int *Dl = Dg + (int64_t)layer * E * E;
         long long acc = 0;
@@ -252,7 +256,7 @@ int loss_blocks_per_problem(const Problem &p) {
     return (int)(blocks < 1 ? 1 : blocks);
 }
 
-WsLayout ws_layout(const Problem &p) {
+WsLayout ws_layout(const Problem &p, bool wide) {
     auto up = [](size_t x) { return (x + 255) / 256 * 256; };
     WsLayout w;
     const int64_t fast_parts = p.W;  // the fast kernel gives every CTA at least 32 tokens
@@ -260,20 +264,22 @@ WsLayout ws_layout(const Problem &p) {
     w.max_parts = (int)(fast_parts > gen_parts ? fast_parts : gen_parts);
     const bool fast_k = p.k == 1 || p.k == 2 || p.k == 4 || p.k == 8;
     const bool fast_e = p.E == 32 || p.E == 64 || p.E == 128;
+    w.cooc = (fast_k && fast_e) || (wide && cooc_sizes_ok(p.E, p.k));
+    w.image = w.cooc && (wide ? bimg_sizes_ok(p.E, p.k) : p.E == 128);
     w.done = kWsHeader;
     w.partials = up(w.done + sizeof(int) * (size_t)p.L);
     w.idx = up(w.partials + sizeof(double) * (size_t)p.L * (size_t)w.max_parts);
     w.cooc_parts = up(w.idx + (fast_k ? (size_t)p.L * (size_t)p.T * (size_t)p.k : 0));
-    const size_t parts = (fast_k && fast_e) ? sizeof(uint32_t) * (size_t)p.L *
+    const size_t parts = w.cooc ? sizeof(uint32_t) * (size_t)p.L *
                                                   (size_t)max_sig_ctas_per_problem(p) *
                                                   cooc_partial_words(p.E)
                                             : 0;
     w.n_acc = up(w.cooc_parts + parts);
-    w.bimg = up(w.n_acc + ((fast_k && fast_e) ? sizeof(int) * (size_t)p.L * p.E : 0));
+    w.bimg = up(w.n_acc + (w.cooc ? sizeof(int) * (size_t)p.L * p.E : 0));
     // the dispatch order of a routed call may run beside the loss kernel: its
     // scratch has a region of its own
-    w.img_ok = up(w.bimg + ((fast_k && p.E == 128) ? (size_t)kBImageBytes * (size_t)p.L : 0));
-    w.route_base = up(w.img_ok + ((fast_k && p.E == 128) ? sizeof(int) * (size_t)p.L : 0));
+    w.img_ok = up(w.bimg + (w.image ? (size_t)bimg_bytes(cooc_width(p.E)) * (size_t)p.L : 0));
+    w.route_base = up(w.img_ok + (w.image ? sizeof(int) * (size_t)p.L : 0));
     w.total = up(w.route_base + sizeof(int) * (size_t)route_scratch_ints(p));
     return w;
 }
@@ -286,10 +292,8 @@ int max_sig_ctas_per_problem(const Problem &p) {
 
 cudaError_t launch_loss(const float *logits, const uint32_t *bits, const int *D, const Problem &p,
                         int gate, float d_scale, float grad_scale, float *loss,
-                        long long *origin_do, float *dlogits, void *workspace, cudaStream_t s) {
-    int *status = reinterpret_cast<int *>(workspace);
-    double *partials =
-        reinterpret_cast<double *>(static_cast<char *>(workspace) + ws_layout(p).partials);
+                        long long *origin_do, float *dlogits, int *status, double *partials,
+                        cudaStream_t s, int *n_zero) {
     const int P = loss_blocks_per_problem(p);
     const double norm = 1.0 / ((double)p.T * (double)p.T * (double)p.k);
     const float coef = (float)((double)grad_scale * (double)d_scale * norm);
@@ -303,7 +307,7 @@ cudaError_t launch_loss(const float *logits, const uint32_t *bits, const int *D,
     else e = dispatch_gate<32>(logits, bits, D, p, gate, coef, dlogits, partials, P, status, s);
     if (e != cudaSuccess) return e;
     loss_finalize_kernel<<<p.L, 256, 0, s>>>(partials, P, D, p.E, (double)d_scale * norm, loss,
-                                             origin_do);
+                                             origin_do, n_zero);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,8 @@
+// The tensor-core loss kernel at 4 boxes of 32 experts.
+#include "loss_mma.cuh"
+
+namespace dol {
+
+DOL_LOSS_MMA_INSTANCE(4)
+
+}  // namespace dol

@@ -2,9 +2,9 @@
 // probabilities, only the K chosen ones and re-normalizes them; these weigh
 // the chosen experts' outputs.  The selection pass that builds the signatures
 // writes the chosen experts and those weights (the kRoute instantiations of
-// the kernel in sig_fast.cuh, or the generic kernel); this file launches them
-// and holds the two dispatch kernels, which put the routed (token, choice)
-// pairs in expert order:
+// the kernel in sig_fast.cuh, select.cuh or the generic kernel); this file
+// launches the first and holds the two dispatch kernels, which put the routed
+// (token, choice) pairs in expert order:
 //   offsets[e] = n_0 + ... + n_{e-1}, offsets[E] = T k
 //   rows[offsets[e] + r] = the r-th token (ascending) routed to expert e
 //   pos[t][q] = the row of the pair (t, q), so rows[pos[t][q]] = t.

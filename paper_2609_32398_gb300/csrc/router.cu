@@ -44,12 +44,12 @@ constexpr int kREpiWarps = 4;
 constexpr int kRThreads = (2 + kREpiWarps) * 32;
 constexpr int kRZTileBytes = 32 * kRE * 4;      // one warp's 32 tokens x 128 logits
 constexpr int kRTmemCols = 4 * kRE;             // two buffers x two fp32 accumulators
-using RC = SigCfg<kRE>;
+constexpr int kRTriWords = tri_words(kRE);
 
 constexpr size_t kROffZ = (size_t)kRStages * kRStageBytes;
-constexpr size_t kROffRowoff = kROffZ + (size_t)kREpiWarps * kRZTileBytes;
-constexpr size_t kROffTri = kROffRowoff + (size_t)kRE * 4;          // packed 16-bit counters
-constexpr size_t kROffBars = kROffTri + (size_t)(RC::kCoocWords / 2) * 4;
+constexpr size_t kROffColoff = kROffZ + (size_t)kREpiWarps * kRZTileBytes;
+constexpr size_t kROffTri = kROffColoff + (size_t)kRE * 4;          // packed 16-bit counters
+constexpr size_t kROffBars = kROffTri + (size_t)(kRTriWords / 2) * 4;
 constexpr size_t kRNumBars = 2 * kRStages + 4;
 constexpr size_t kROffScal = kROffBars + kRNumBars * 8;
 constexpr size_t kRSmem = kROffScal + 16 + 1024;  // + alignment slack of the base
@@ -80,7 +80,7 @@ router_sig_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constan
     unsigned char *smem = smem_align<1024>(smem_raw);
     unsigned char *ring = smem;
     unsigned char *ztiles = smem + kROffZ;
-    int *s_rowoff = reinterpret_cast<int *>(smem + kROffRowoff);
+    int *s_coloff = reinterpret_cast<int *>(smem + kROffColoff);
     uint32_t *s_tri = reinterpret_cast<uint32_t *>(smem + kROffTri);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kROffBars);
     uint64_t *full = bars, *empty = bars + kRStages;
@@ -96,12 +96,12 @@ router_sig_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constan
     const int64_t wb = (int64_t)blockIdx.x * a.W / gridDim.x;
     const int64_t we = (int64_t)(blockIdx.x + 1) * a.W / gridDim.x;
     // this CTA's co-occurrence triangle (the reduction kernel's input)
-    uint32_t *tri = a.cooc + ((size_t)layer * gridDim.x + blockIdx.x) * (size_t)RC::kCoocWords;
+    uint32_t *tri = a.cooc + ((size_t)layer * gridDim.x + blockIdx.x) * (size_t)kRTriWords;
     // Shared-memory and TMEM set-up touch no global memory: they overlap the
     // end of the previous kernel on the stream.
-    for (int e = threadIdx.x; e < kRE; e += kRThreads) s_rowoff[e] = cooc_row_offset<kRE>(e) - (e & ~3);
+    for (int e = threadIdx.x; e < kRE; e += kRThreads) s_coloff[e] = tri_chunk(e >> 2) + (e & 3);
     if (a.packed)
-        for (int i = threadIdx.x; i < RC::kCoocWords / 2; i += kRThreads) s_tri[i] = 0u;
+        for (int i = threadIdx.x; i < kRTriWords / 2; i += kRThreads) s_tri[i] = 0u;
     if (threadIdx.x == 0) {
         for (int s = 0; s < kRStages; ++s) {
             mbar_init(&full[s], 1);
@@ -134,7 +134,7 @@ router_sig_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constan
             a.zero.p[z][i] = 0;
     if (!a.packed) {  // the global triangle starts at zero (ordered by the barrier)
         uint4 *t4 = reinterpret_cast<uint4 *>(tri);
-        for (int q = threadIdx.x; q < RC::kCoocWords / 4; q += kRThreads) t4[q] = make_uint4(0u, 0u, 0u, 0u);
+        for (int q = threadIdx.x; q < kRTriWords / 4; q += kRThreads) t4[q] = make_uint4(0u, 0u, 0u, 0u);
     }
     __syncthreads();
 
@@ -274,10 +274,10 @@ router_sig_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constan
                         }
 #pragma unroll
                     for (int q1 = 0; q1 < K - 1; ++q1) {
-                        const int row = s_rowoff[so[q1]];
+                        const int row = 4 * so[q1];
 #pragma unroll
                         for (int q2 = q1 + 1; q2 < K; ++q2) {
-                            const int wi = row + so[q2];
+                            const int wi = row + s_coloff[so[q2]];
                             if (a.packed) atomicAdd(&s_tri[wi >> 1], 1u << (16 * (wi & 1)));
                             else atomicAdd(&tri[wi], 1u);
                         }
@@ -293,7 +293,7 @@ router_sig_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constan
         for (int r = 0; r < kRE / 32; ++r)
             if (cnt[r]) {
                 const int e = 32 * r + lane;
-                const int wi = s_rowoff[e] + e;
+                const int wi = s_coloff[e] + 4 * e;
                 if (a.packed) atomicAdd(&s_tri[wi >> 1], cnt[r] << (16 * (wi & 1)));
                 else atomicAdd(&tri[wi], cnt[r]);
                 atomicAdd(&a.counts[layer * kRE + e], (int)cnt[r]);
@@ -301,7 +301,7 @@ router_sig_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constan
         if (a.packed) {
             // all epilogue warps have counted: the triangle out, unpacked
             asm volatile("bar.sync 1, %0;" ::"n"(kREpiWarps * 32) : "memory");
-            for (int q = threadIdx.x - 64; q < RC::kCoocWords / 2; q += kREpiWarps * 32) {
+            for (int q = threadIdx.x - 64; q < kRTriWords / 2; q += kREpiWarps * 32) {
                 const uint32_t v = s_tri[q];
                 reinterpret_cast<uint2 *>(tri)[q] = make_uint2(v & 0xFFFFu, v >> 16);
             }

@@ -1,5 +1,5 @@
-// Step 1, fast path (E in {32, 64, 128, 256}, k in {1, 2, 4, 8}, 16-byte
-// aligned logits; at E = 256 without the co-occurrence counts): Top-K
+// Step 1 for E in {32, 64, 128} and k in {1, 2, 4, 8} (16-byte aligned logits;
+// the other sizes take the kernel of select.cuh): Top-K
 // signatures (Sec. 3.1.1, Eq. 1) with one token per lane.
 //
 // A persistent CTA per SM owns a contiguous range of 32-token tiles.  One
@@ -44,12 +44,11 @@ template <int E>
 struct SigCfg {
     static constexpr int kBoxes = E / 32;
     static constexpr int kTileBytes = kBoxes * kBoxBytes;
-    static constexpr int kSlots = (E == 256) ? 6 : (E == 128) ? 11 : 16;
+    static constexpr int kSlots = (E == 128) ? 11 : 16;
     static constexpr int GS = (E >= 128) ? E / 16 : 4;  // experts per group
     static constexpr int NG = E / GS;                    // groups per row
-    // co-occurrence counters: row a holds columns (a & ~3) .. E-1 (E <= 128;
-    // at E = 256 the kernel runs without them)
-    static constexpr int kCoocWords = E <= 128 ? cooc_row_offset<E>(E) : 0;
+    // co-occurrence counters in the triangle of tri_chunk
+    static constexpr int kCoocWords = tri_words(E);
     static constexpr size_t kSmem = (size_t)kSlots * kTileBytes + 1024 + 2 * kSlots * 8 +
                                     kSlots * 4 + 32 + (size_t)kCoocWords * 4 + E * 4 +
                                     (size_t)kConsumers * E * 4;
@@ -233,19 +232,19 @@ __device__ __forceinline__ void sort_small(int (&so)[K]) {
 }
 
 // c_ab += 1 for every pair a < b of one token's chosen experts, in a
-// shared-memory triangle whose row a starts at s_rowoff[a] (the counts on the
-// diagonal come from the signature words).
+// shared-memory triangle whose column b starts at s_coloff[b] (the counts on
+// the diagonal come from the signature words).
 template <int K>
-__device__ __forceinline__ void cooc_add(uint32_t *s_cooc, const int *s_rowoff, const int (&sel)[K]) {
+__device__ __forceinline__ void cooc_add(uint32_t *s_cooc, const int *s_coloff, const int (&sel)[K]) {
     int so[K];
 #pragma unroll
     for (int q = 0; q < K; ++q) so[q] = sel[q];
     sort_small<K>(so);
 #pragma unroll
-    for (int q1 = 0; q1 < K - 1; ++q1) {
-        uint32_t *row = s_cooc + s_rowoff[so[q1]];
+    for (int q2 = 1; q2 < K; ++q2) {
+        uint32_t *col = s_cooc + s_coloff[so[q2]];
 #pragma unroll
-        for (int q2 = q1 + 1; q2 < K; ++q2) atomicAdd(row + so[q2], 1u);
+        for (int q1 = 0; q1 < q2; ++q1) atomicAdd(col + 4 * so[q1], 1u);
     }
 }
 
@@ -318,23 +317,21 @@ sig_fast_kernel(const __grid_constant__ CUtensorMap tmap, int64_t T, int64_t W,
     volatile int *s_abort = slot_round + C::kSlots;
     uint32_t *s_cooc = reinterpret_cast<uint32_t *>(
         smem_align<16>(reinterpret_cast<unsigned char *>(const_cast<int *>(s_abort + 1))));
-    int *s_rowoff = reinterpret_cast<int *>(s_cooc + C::kCoocWords);
-    uint32_t *s_wsc = reinterpret_cast<uint32_t *>(s_rowoff + E);  // [consumer warp][E]
+    int *s_coloff = reinterpret_cast<int *>(s_cooc + C::kCoocWords);
+    uint32_t *s_wsc = reinterpret_cast<uint32_t *>(s_coloff + E);  // [consumer warp][E]
 
     pdl_trigger();
     // this CTA: layer blockIdx.y, a contiguous range of its 32-token tiles
     const int64_t layer = blockIdx.y;
-    const int64_t per = (W + gridDim.x - 1) / gridDim.x;
-    const int64_t tb = (int64_t)blockIdx.x * per;
-    const int64_t te = min64(W, tb + per);
-    const int n = te > tb ? (int)(te - tb) : 0;
+    const int64_t tb = W * (int64_t)blockIdx.x / gridDim.x;
+    const int n = (int)(W * (int64_t)(blockIdx.x + 1) / gridDim.x - tb);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // Shared-memory set-up first: it touches no global memory, so it overlaps
     // the end of the previous kernel on the stream.
     for (int i = threadIdx.x; i < kConsumers * E; i += blockDim.x) s_wsc[i] = 0u;
     if (kCooc) {
         for (int i = threadIdx.x; i < C::kCoocWords; i += blockDim.x) s_cooc[i] = 0u;
-        for (int a = threadIdx.x; a < E; a += blockDim.x) s_rowoff[a] = cooc_row_offset<E>(a) - (a & ~3);
+        for (int a = threadIdx.x; a < E; a += blockDim.x) s_coloff[a] = tri_chunk(a >> 2) + (a & 3);
     }
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::kSlots; ++s) {
@@ -425,7 +422,7 @@ sig_fast_kernel(const __grid_constant__ CUtensorMap tmap, int64_t T, int64_t W,
 
         if (idx && valid) store_idx<K>(idx + (layer * T + t) * K, sel);
         if (kRoute && valid) store_route<K>(route, (layer * T + t) * K, sel, val);
-        if (kCooc && valid) cooc_add<K>(s_cooc, s_rowoff, sel);
+        if (kCooc && valid) cooc_add<K>(s_cooc, s_coloff, sel);
         emit_words_or<E, K, kCounts || kCooc>(sel, valid, lane, s_wsc + warp * E,
                                              bits + layer * E * W + w, W, cnt);
     }
@@ -437,7 +434,7 @@ sig_fast_kernel(const __grid_constant__ CUtensorMap tmap, int64_t T, int64_t W,
     if (kCooc) {  // counts n_a on the triangle's diagonal
 #pragma unroll
         for (int r = 0; r < R; ++r)
-            if (cnt[r]) atomicAdd(&s_cooc[s_rowoff[32 * r + lane] + 32 * r + lane], cnt[r]);
+            if (cnt[r]) atomicAdd(&s_cooc[s_coloff[32 * r + lane] + 4 * (32 * r + lane)], cnt[r]);
     }
     if (kCooc) {
         // all consumer warps have counted: store this CTA's triangle for the
@@ -450,7 +447,7 @@ sig_fast_kernel(const __grid_constant__ CUtensorMap tmap, int64_t T, int64_t W,
         // the diagonal holds this CTA's counts n_a: add them to the layer's totals
         // (counts points at the workspace accumulator on this path)
         for (int a = threadIdx.x; a < E; a += kConsumers * 32) {
-            const uint32_t na = s_cooc[s_rowoff[a] + a];
+            const uint32_t na = s_cooc[s_coloff[a] + 4 * a];
             if (na) atomicAdd(&counts[layer * E + a], (int)na);
         }
     }
@@ -465,7 +462,7 @@ cudaError_t run_fast(const CUtensorMap &map, const Problem &p, uint32_t *bits, i
     cudaError_t e = ensure_smem_limit<sig_fast_kernel<E, K, kCounts, kCooc, kRoute>>(C::kSmem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)sig_fast_ctas_per_problem(p), (unsigned)p.L);
+    cfg.gridDim = dim3((unsigned)sig_ctas_per_problem(p), (unsigned)p.L);
     cfg.blockDim = dim3(kFastThreads);
     cfg.dynamicSmemBytes = C::kSmem;
     cfg.stream = s;

@@ -114,7 +114,7 @@ extern "C" do_status do_forward_backward_static(const float *logits, int64_t T, 
     p.L = L;
     p.W = (T + 31) / 32;
     // no routing outputs here: the layout up to the routing scratch
-    if (dol::workspace_bytes_plain(p) > DO_STATIC_SCRATCH_BYTES) return DO_ERR_WORKSPACE;
+    if (dol::workspace_bytes_plain(p, false) > DO_STATIC_SCRATCH_BYTES) return DO_ERR_WORKSPACE;
     if (!logits || !bits || !counts || !D || !loss) return DO_ERR_INVALID_ARG;
     if (status_flags && reinterpret_cast<uintptr_t>(status_flags) % 4 != 0)
         return DO_ERR_INVALID_ARG;
@@ -128,7 +128,7 @@ extern "C" do_status do_forward_backward_static(const float *logits, int64_t T, 
     // clearing them here also recovers from a call that gave up on a wait.
     // Everything else in the array is written before it is read (the image
     // of D' at bimg by the reduction kernel, every entry of it).
-    const dol::WsLayout w = dol::ws_layout(p);
+    const dol::WsLayout w = dol::ws_layout_for(p, DO_STATIC_SCRATCH_BYTES, true);
     char *base = static_cast<char *>(ws);
     if (cudaMemsetAsync(base, 0, w.partials, s) != cudaSuccess) return DO_ERR_CUDA;
     if (w.bimg > w.n_acc && cudaMemsetAsync(base + w.n_acc, 0, w.bimg - w.n_acc, s) != cudaSuccess)

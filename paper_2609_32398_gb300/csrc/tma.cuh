@@ -108,6 +108,12 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 bool encode_tensor_map_2d_f32(CUtensorMap *map, const float *base, uint64_t rows, uint64_t cols,
                               uint32_t box_rows);
 
+// Host: the same tensor (cols a multiple of 32) seen as [cols / 32][rows][32],
+// box cols / 32 x box_rows x 32: the 2-D boxes of a row range one after the
+// other in shared memory, in one copy.
+bool encode_tensor_map_boxes_f32(CUtensorMap *map, const float *base, uint64_t rows, uint64_t cols,
+                                 uint32_t box_rows);
+
 }  // namespace dol
 
 namespace dol {

@@ -38,6 +38,20 @@ bool encode_tensor_map_2d_f32(CUtensorMap *map, const float *base, uint64_t rows
     return r == CUDA_SUCCESS;
 }
 
+bool encode_tensor_map_boxes_f32(CUtensorMap *map, const float *base, uint64_t rows, uint64_t cols,
+                                 uint32_t box_rows) {
+    PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
+    if (!fn || cols % 32 != 0) return false;
+    const cuuint64_t dims[3] = {32, rows, cols / 32};
+    const cuuint64_t strides[2] = {cols * sizeof(float), 32 * sizeof(float)};
+    const cuuint32_t box[3] = {32, box_rows, (cuuint32_t)(cols / 32)};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float *>(base), dims, strides,
+                    box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS;
+}
+
 bool encode_tensor_map_3d_f32(CUtensorMap *map, const float *base, uint64_t planes, uint64_t rows,
                               uint64_t cols, uint32_t box_rows) {
     PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
