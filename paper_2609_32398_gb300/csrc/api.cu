@@ -187,7 +187,7 @@ do_status do_loss_fwd_bwd(const float *logits, const uint32_t *bits, const int32
         int *img_ok = reinterpret_cast<int *>(ws + w.img_ok);
         e = dol::launch_dprime_image(D, p, bimg, img_ok, origin, done, s);
         if (e == cudaSuccess)
-            e = dol::launch_loss_mma(logits, bits, bimg, nullptr, p, gate, d_scale, grad_scale, loss,
+            e = dol::launch_loss_mma(logits, bits, nullptr, bimg, nullptr, p, gate, d_scale, grad_scale, loss,
                                      dlogits, partials, done, status, nullptr, s, nullptr, nullptr,
                                      img_ok, D);
         return from_cuda(e);
@@ -245,7 +245,9 @@ do_status forward_backward_impl(const float *logits, int64_t T, int32_t E, int32
                           (dol::loss_fast_supported(p, logits, D, dlogits) ||
                            dol::loss_fast256_supported(p, logits, D, dlogits));
     const bool mma = select && w.image && dol::loss_mma_supported(p, logits, dlogits);
-    uint8_t *idx = loss_idx && !mma ? reinterpret_cast<uint8_t *>(ws + w.idx) : nullptr;
+    // (the tensor-core one where it is cheap for the selection to write them)
+    const bool use_idx = loss_idx && (!mma || dol::signatures_fast_supported(logits, p));
+    uint8_t *idx = use_idx ? reinterpret_cast<uint8_t *>(ws + w.idx) : nullptr;
     // the router GEMM runs only in the fused fast path, without routing outputs
     if (rin && !(loss_idx && w.cooc && !ra &&
                  dol::router_supported(p, rin->H, rin->X, rin->Wr, logits)))
@@ -272,7 +274,7 @@ do_status forward_backward_impl(const float *logits, int64_t T, int32_t E, int32
         if (e == cudaSuccess)
             e = dol::launch_cooc_reduce(parts, P1, n_acc, p, D, counts, bimg, big, origin, s);
         if (e == cudaSuccess && mma) {
-            e = dol::launch_loss_mma(logits, bits, bimg, n_acc, p, gate, 1.0f, grad_scale, loss, dlogits,
+            e = dol::launch_loss_mma(logits, bits, idx, bimg, n_acc, p, gate, 1.0f, grad_scale, loss, dlogits,
                                      partials, done, status, status_out, s);
             if (e == cudaSuccess && status_done) *status_done = status_out != nullptr;
             if (e == cudaSuccess && ra)
@@ -405,7 +407,9 @@ do_status do_routed_forward(const float *logits, int64_t T, int32_t E, int32_t k
         // what the backward half's loss kernel reads
         unsigned char *bimg = split_mma(p, logits, w)
                                   ? reinterpret_cast<unsigned char *>(ws + w.bimg) : nullptr;
-        const dol::SelectOut so = {bits, n_acc, nullptr, parts, zero, reinterpret_cast<int *>(ws), route};
+        uint8_t *idx = dol::signatures_fast_supported(logits, p)
+                           ? reinterpret_cast<uint8_t *>(ws + w.idx) : nullptr;
+        const dol::SelectOut so = {bits, n_acc, idx, parts, zero, reinterpret_cast<int *>(ws), route};
         e = dol::launch_select(logits, p, so, s);
         if (e == cudaSuccess)
             e = dol::launch_cooc_reduce(parts, dol::sig_ctas_per_problem(p), n_acc, p, D,
@@ -467,9 +471,10 @@ do_status do_routed_backward(const float *logits, int64_t T, int32_t E, int32_t 
         e = local ? cudaSuccess : dol::launch_dprime_image(D, p, bimg, img_ok, nullptr, nullptr, s);
         // the routing gradient is added in the loss kernel's epilogue where it
         // can, else by its own kernel
-        const bool rg_mma = rg && dol::loss_mma_route_grad(p, gate, expert_ids, grad_combine);
+        const bool have_idx = dol::signatures_fast_supported(logits, p);
+        const bool rg_mma = rg && have_idx && dol::loss_mma_route_grad(p, gate, expert_ids, grad_combine);
         if (e == cudaSuccess)
-            e = dol::launch_loss_mma(logits, bits, bimg, local ? n_acc : nullptr, p, gate, d_scale,
+            e = dol::launch_loss_mma(logits, bits, have_idx ? idx : nullptr, bimg, local ? n_acc : nullptr, p, gate, d_scale,
                                      grad_scale, loss, dlogits, partials, done, status, nullptr, s,
                                      rg_mma ? expert_ids : nullptr, rg_mma ? grad_combine : nullptr,
                                      img_ok, local ? nullptr : D);

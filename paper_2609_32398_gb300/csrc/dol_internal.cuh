@@ -196,8 +196,10 @@ cudaError_t launch_idx_from_bits(const uint32_t *bits, const Problem &p, uint8_t
 bool loss_mma_supported(const Problem &p, const float *logits, const float *dlogits);
 bool loss_mma_big(const Problem &p);
 bool loss_mma_route_grad(const Problem &p, int gate, const int *ids, const float *g);
-cudaError_t launch_loss_mma(const float *logits, const uint32_t *bits, const unsigned char *bimg,
-                            int *n_zero, const Problem &p, int gate, float d_scale, float grad_scale,
+// idx (may be null; k in {1, 2, 4, 8}, E in {32, 64, 128}; needed for the routing
+// gradient): the chosen experts of every token, as the selection wrote them.
+cudaError_t launch_loss_mma(const float *logits, const uint32_t *bits, const uint8_t *idx,
+                            const unsigned char *bimg, int *n_zero, const Problem &p, int gate, float d_scale, float grad_scale,
                             float *loss, float *dlogits, double *partials, int *done, int *status,
                             int *status_out, cudaStream_t s, const int *rg_ids = nullptr,
                             const float *rg_g = nullptr, const int *img_ok = nullptr,

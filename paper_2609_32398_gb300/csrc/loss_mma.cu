@@ -4,10 +4,10 @@
 
 namespace dol {
 
-template <> cudaError_t run_loss_mma<1>(const CUtensorMap &, const CUtensorMap &, const MmaArgs &, int, bool, bool, int, int, cudaStream_t);
-template <> cudaError_t run_loss_mma<2>(const CUtensorMap &, const CUtensorMap &, const MmaArgs &, int, bool, bool, int, int, cudaStream_t);
-template <> cudaError_t run_loss_mma<3>(const CUtensorMap &, const CUtensorMap &, const MmaArgs &, int, bool, bool, int, int, cudaStream_t);
-template <> cudaError_t run_loss_mma<4>(const CUtensorMap &, const CUtensorMap &, const MmaArgs &, int, bool, bool, int, int, cudaStream_t);
+template <> cudaError_t run_loss_mma<1>(const CUtensorMap &, const CUtensorMap &, const MmaArgs &, int, bool, bool, bool, int, int, cudaStream_t);
+template <> cudaError_t run_loss_mma<2>(const CUtensorMap &, const CUtensorMap &, const MmaArgs &, int, bool, bool, bool, int, int, cudaStream_t);
+template <> cudaError_t run_loss_mma<3>(const CUtensorMap &, const CUtensorMap &, const MmaArgs &, int, bool, bool, bool, int, int, cudaStream_t);
+template <> cudaError_t run_loss_mma<4>(const CUtensorMap &, const CUtensorMap &, const MmaArgs &, int, bool, bool, bool, int, int, cudaStream_t);
 
 namespace {
 
@@ -36,12 +36,12 @@ bool loss_mma_route_grad(const Problem &p, int gate, const int *ids, const float
     return p.E == 128 && gate == 0 && k_ok && al(ids) && al(g);
 }
 
-cudaError_t launch_loss_mma(const float *logits, const uint32_t *bits, const unsigned char *bimg,
-                            int *n_zero, const Problem &p, int gate, float d_scale, float grad_scale,
+cudaError_t launch_loss_mma(const float *logits, const uint32_t *bits, const uint8_t *idx,
+                            const unsigned char *bimg, int *n_zero, const Problem &p, int gate, float d_scale, float grad_scale,
                             float *loss, float *dlogits, double *partials, int *done, int *status,
                             int *status_out, cudaStream_t s, const int *rg_ids, const float *rg_g,
                             const int *img_ok, const int *D) {
-    if (!bimg || (img_ok && !D) || (rg_ids && !loss_mma_route_grad(p, gate, rg_ids, rg_g)))
+    if (!bimg || (img_ok && !D) || (rg_ids && (!idx || !loss_mma_route_grad(p, gate, rg_ids, rg_g))))
         return cudaErrorInvalidValue;
     CUtensorMap zmap, dzmap;
     if (!encode_tensor_map_3d_f32(&zmap, logits, (uint64_t)p.L, (uint64_t)p.T, (uint64_t)p.E, 32))
@@ -56,6 +56,8 @@ cudaError_t launch_loss_mma(const float *logits, const uint32_t *bits, const uns
     const double norm = 1.0 / ((double)p.T * (double)p.T * (double)p.k);
     MmaArgs args;
     args.bits = bits;
+    args.idx = idx;
+    args.k = p.k;
     args.bimg = bimg;
     args.n_zero = n_zero;
     args.T = p.T;
@@ -79,8 +81,8 @@ cudaError_t launch_loss_mma(const float *logits, const uint32_t *bits, const uns
     const bool big = img_ok != nullptr || loss_mma_big(p);
     if (rg_ids && rg_g) {
 #define DOL_RG_CASE(KK)                                                                       \
-    return big ? run_mma<4, 0, true, false, KK>(zmap, dzmap, args, (int)gx, p.L, s)          \
-               : run_mma<4, 0, false, false, KK>(zmap, dzmap, args, (int)gx, p.L, s)
+    return big ? run_mma<4, 0, true, false, true, KK>(zmap, dzmap, args, (int)gx, p.L, s)          \
+               : run_mma<4, 0, false, false, true, KK>(zmap, dzmap, args, (int)gx, p.L, s)
         switch (p.k) {
             case 1: DOL_RG_CASE(1);
             case 2: DOL_RG_CASE(2);
@@ -91,10 +93,10 @@ cudaError_t launch_loss_mma(const float *logits, const uint32_t *bits, const uns
     }
     const bool pad = p.E % 32 != 0;
     switch (cooc_width(p.E) / 32) {
-        case 1: return run_loss_mma<1>(zmap, dzmap, args, gate, big, pad, (int)gx, p.L, s);
-        case 2: return run_loss_mma<2>(zmap, dzmap, args, gate, big, pad, (int)gx, p.L, s);
-        case 3: return run_loss_mma<3>(zmap, dzmap, args, gate, big, pad, (int)gx, p.L, s);
-        default: return run_loss_mma<4>(zmap, dzmap, args, gate, big, pad, (int)gx, p.L, s);
+        case 1: return run_loss_mma<1>(zmap, dzmap, args, gate, big, pad, idx != nullptr, (int)gx, p.L, s);
+        case 2: return run_loss_mma<2>(zmap, dzmap, args, gate, big, pad, idx != nullptr, (int)gx, p.L, s);
+        case 3: return run_loss_mma<3>(zmap, dzmap, args, gate, big, pad, idx != nullptr, (int)gx, p.L, s);
+        default: return run_loss_mma<4>(zmap, dzmap, args, gate, big, pad, idx != nullptr, (int)gx, p.L, s);
     }
 }
 
