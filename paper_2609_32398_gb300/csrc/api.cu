@@ -302,7 +302,7 @@ do_status forward_backward_impl(const float *logits, int64_t T, int32_t E, int32
             if (e == cudaSuccess && status_done) *status_done = status_out != nullptr;
         } else {
             e = dol::launch_loss(logits, bits, D, p, gate, 1.0f, grad_scale, loss, origin, dlogits,
-                                 status, partials, s, n_acc);
+                                 status, partials, s, counts, n_acc);
         }
     }
     // the dispatch order (from the signatures and ids alone) follows the loss kernel
@@ -488,7 +488,7 @@ do_status do_routed_backward(const float *logits, int64_t T, int32_t E, int32_t 
                                       status, nullptr, s);
     } else {
         e = dol::launch_loss(logits, bits, D, p, gate, d_scale, grad_scale, loss, nullptr, dlogits,
-                             status, partials, s);
+                             status, partials, s, local ? counts : nullptr);
     }
     // elsewhere the routing gradient is added by its own kernel
     if (e == cudaSuccess && rg)

@@ -98,8 +98,8 @@ inline WsLayout ws_layout_for(const Problem &p, size_t bytes, bool plain) {
     return (plain ? w.route_base : w.total) <= bytes ? w : ws_layout(p, false);
 }
 
-// Number of generic loss-kernel CTAs per problem; fixes the partial-sum
-// layout and therefore the reduction order.
+// Partial-sum slots per problem that the workspace has at least (with W if that
+// is more).
 int loss_blocks_per_problem(const Problem &p);
 
 // Launchers (return the first CUDA error, cudaSuccess otherwise).
@@ -144,11 +144,13 @@ cudaError_t launch_origin_do(const int *D, const Problem &p, long long *origin_d
 // local Hamming matrix from its origin_do (App. C.1).
 cudaError_t launch_offdiag_variance(const long long *origin_do, const Problem &p, double *var,
                                     cudaStream_t s);
-// Generic loss (any E, k): n_zero ([L][E], may be null) is cleared.
+// Generic loss (any E, k).  counts (may be null): n_i of the same tokens, D being
+// their own matrix; n_zero ([L][E], may be null) is cleared.
 cudaError_t launch_loss(const float *logits, const uint32_t *bits, const int *D,
                         const Problem &p, int gate, float d_scale, float grad_scale,
                         float *loss, long long *origin_do, float *dlogits, int *status,
-                        double *partials, cudaStream_t s, int *n_zero = nullptr);
+                        double *partials, cudaStream_t s, const int *counts = nullptr,
+                        int *n_zero = nullptr);
 
 // Dispatch order of the routed (token, choice) pairs from the signatures and
 // the chosen ids alone: offsets [L][E+1], rows [L][T k], pos [L][T][k] (each

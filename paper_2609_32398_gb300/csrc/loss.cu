@@ -21,8 +21,6 @@
 namespace dol {
 namespace {
 
-constexpr int kLossThreads = 256;
-constexpr int kLossWarps = kLossThreads / 32;
 constexpr size_t kSmemDLimit = 200 * 1024;
 
 __device__ __forceinline__ float sigmoid_f(float z) {
@@ -31,14 +29,26 @@ __device__ __forceinline__ float sigmoid_f(float z) {
     return __fdividef(1.0f, 1.0f + e);
 }
 
+// Warps per CTA: fewer where a lane holds many experts (registers).
+template <int R>
+constexpr int loss_warps() { return R <= 8 ? 16 : 8; }
+constexpr int kListMax = 64;  // chosen experts of a token listed in shared memory
+
+// A warp per token: lanes hold experts i = lane + 32 r (r < R).  The tokens of a
+// signature word are split over `split` warps (a power of two), so that a short
+// window still fills the GPU: with 32 tokens in turn per warp the kernel took
+// 170 of 202 us at E = 200, T = 2539.  The k chosen rows of D are read four at
+// a time.
 template <int R, bool kSmemD, int kGate>
-__global__ void __launch_bounds__(kLossThreads)
+__global__ void __launch_bounds__(loss_warps<R>() * 32)
 loss_generic_kernel(const float *__restrict__ logits, const uint32_t *__restrict__ bits,
-                    const int *__restrict__ Dg, int64_t T, int E, int64_t W, float coef,
-                    float *__restrict__ dlogits, double *__restrict__ partials, int P,
-                    int *__restrict__ status) {
+                    const int *__restrict__ Dg, const int *__restrict__ counts, int64_t T, int E, int k,
+                    int64_t W, int split, float coef, float *__restrict__ dlogits,
+                    double *__restrict__ partials, int P, int *__restrict__ status) {
+    constexpr int kLossWarps = loss_warps<R>();
     extern __shared__ __align__(16) int smem[];
     __shared__ double s_part[kLossWarps];
+    __shared__ int s_list[kLossWarps][kListMax];
     int *sD = smem;
     int *sR = smem + (kSmemD ? E * E : 0);
 
@@ -48,13 +58,27 @@ loss_generic_kernel(const float *__restrict__ logits, const uint32_t *__restrict
     float *dz = dlogits ? dlogits + (int64_t)layer * T * E : nullptr;
     const uint32_t *bl = bits + (int64_t)layer * E * W;
 
-    if (kSmemD)
-        for (int idx = threadIdx.x; idx < E * E; idx += blockDim.x) sD[idx] = __ldg(Dl + idx);
-    __syncthreads();
+    if (kSmemD) {
+        if ((E & 3) == 0 && (reinterpret_cast<uintptr_t>(Dl) & 15) == 0) {
+#pragma unroll 4
+            for (int q = threadIdx.x; q < E * E / 4; q += blockDim.x)
+                reinterpret_cast<int4 *>(sD)[q] = __ldg(reinterpret_cast<const int4 *>(Dl) + q);
+        } else {
+            for (int q = threadIdx.x; q < E * E; q += blockDim.x) sD[q] = __ldg(Dl + q);
+        }
+        __syncthreads();
+    }
     const int *Dsrc = kSmemD ? sD : Dl;
     for (int i = threadIdx.x; i < E; i += blockDim.x) {
+        // R_i = (E - 2k) n_i + T k for the matrix of the same tokens, else a
+        // column sum (D symmetric)
         long long acc = 0;
-        for (int j = 0; j < E; ++j) acc += Dsrc[(int64_t)i * E + j];
+        if (counts) {
+            acc = (long long)(E - 2 * k) * counts[(int64_t)layer * E + i] + (long long)T * k;
+        } else {
+#pragma unroll 8
+            for (int j = 0; j < E; ++j) acc += Dsrc[(int64_t)j * E + i];
+        }
         if (acc > INT_MAX || acc < 0) atomicOr(status, kDevOverflow);
         sR[i] = (int)acc;
     }
@@ -62,52 +86,84 @@ loss_generic_kernel(const float *__restrict__ logits, const uint32_t *__restrict
 
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    int Ri[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int i = lane + 32 * r;
-        Ri[r] = (i < E) ? sR[i] : 0;
-    }
+    int *list = s_list[warp];
     double tok_sum = 0.0;  // sum of A_t over this warp's tokens (meaningful in lane 0)
+    const int per = 32 / split;
 
-    for (int64_t w = (int64_t)blockIdx.x * kLossWarps + warp; w < W;
-         w += (int64_t)P * kLossWarps) {
+    for (int64_t item = (int64_t)blockIdx.x * kLossWarps + warp; item < W * split;
+         item += (int64_t)P * kLossWarps) {
+        const int64_t w = item / split;
+        const int tt0 = (int)(item - w * split) * per;
         uint32_t bw[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int i = lane + 32 * r;
             bw[r] = (i < E) ? __ldg(bl + (int64_t)i * W + w) : 0u;
         }
-        const int64_t t0 = w * 32;
-        const int nt = (int)min64(32, T - t0);
-        for (int tt = 0; tt < nt; ++tt) {
-            const int64_t t = t0 + tt;
+        const int nt = (int)min64(tt0 + per, T - w * 32);
+        for (int tt = tt0; tt < nt; ++tt) {
+            const int64_t t = w * 32 + tt;
             const float *zt = z + t * E;
+            float zr[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int i = lane + 32 * r;
+                zr[r] = (i < E) ? __ldg(zt + i) : 0.0f;
+            }
             int acc[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) acc[r] = 0;
             // sum_{j in S_t} D_ji for this lane's experts i
+            if (k <= kListMax) {
+                int n = 0;
 #pragma unroll
-            for (int rr = 0; rr < R; ++rr) {
-                unsigned m = __ballot_sync(kFull, (bw[rr] >> tt) & 1u);
-                while (m) {
-                    const int j = 32 * rr + __ffs(m) - 1;
-                    m &= m - 1;
-                    const int *row = Dsrc + (int64_t)j * E;
+                for (int rr = 0; rr < R; ++rr) {
+                    const unsigned m = __ballot_sync(kFull, (bw[rr] >> tt) & 1u);
+                    const int at = n + __popc(m & ((1u << lane) - 1u));
+                    if (((m >> lane) & 1u) && at < kListMax) list[at] = 32 * rr + lane;
+                    n += __popc(m);
+                }
+                n = min(n, kListMax);
+                __syncwarp();
+                for (int q = 0; q < n; q += 4) {
+                    const int *row[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) row[u] = Dsrc + (int64_t)list[min(q + u, n - 1)] * E;
 #pragma unroll
                     for (int r = 0; r < R; ++r) {
                         const int i = lane + 32 * r;
-                        if (i < E) acc[r] += row[i];
+                        if (i < E) {
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                const int d = row[u][i];
+                                acc[r] += q + u < n ? d : 0;
+                            }
+                        }
+                    }
+                }
+                __syncwarp();
+            } else {
+#pragma unroll
+                for (int rr = 0; rr < R; ++rr) {
+                    unsigned m = __ballot_sync(kFull, (bw[rr] >> tt) & 1u);
+                    while (m) {
+                        const int j = 32 * rr + __ffs(m) - 1;
+                        m &= m - 1;
+                        const int *row = Dsrc + (int64_t)j * E;
+#pragma unroll
+                        for (int r = 0; r < R; ++r) {
+                            const int i = lane + 32 * r;
+                            if (i < E) acc[r] += row[i];
+                        }
                     }
                 }
             }
-            float zr[R], wr[R], g[R];
+            float wr[R], g[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 const int i = lane + 32 * r;
                 const bool f = (bw[r] >> tt) & 1u;
-                wr[r] = (float)(f ? Ri[r] - acc[r] : -acc[r]);
-                zr[r] = (i < E) ? __ldg(zt + i) : 0.0f;
+                wr[r] = (float)(f ? sR[i] - acc[r] : -acc[r]);
             }
             float num = 0.0f, den = 0.0f;
             if (kGate == 0) {  // sigmoid-norm
@@ -159,68 +215,82 @@ loss_generic_kernel(const float *__restrict__ logits, const uint32_t *__restrict
     }
 }
 
-// loss[l] = d_scale/(m^2 k) * sum of the partials in block order; origin_do[l]
-// = sum_{i != j} D_ij^2 (Eq. origin_do), exact in int64.
+// loss[l] = d_scale/(m^2 k) * sum of the partials in block order.
 __global__ void __launch_bounds__(256)
-loss_finalize_kernel(const double *__restrict__ partials, int P, const int *__restrict__ Dg, int E,
-                     double scale, float *__restrict__ loss, long long *__restrict__ origin_do,
-                     int *__restrict__ n_zero) {
-    __shared__ long long s_red[256];
+loss_finalize_kernel(const double *__restrict__ partials, int P, int E, double scale,
+                     float *__restrict__ loss, int *__restrict__ n_zero) {
     __shared__ double s_dred[256];
     const int layer = blockIdx.x;
-    {
-        const double s = block_sum_fixed(partials + (int64_t)layer * P, P, s_dred, 256);
-        if (threadIdx.x == 0) loss[layer] = (float)(s * scale);
-    }
+    const double s = block_sum_fixed(partials + (int64_t)layer * P, P, s_dred, 256);
+    if (threadIdx.x == 0) loss[layer] = (float)(s * scale);
     // the counts accumulator has been read: cleared for the next call
     if (n_zero)
         for (int i = threadIdx.x; i < E; i += blockDim.x) n_zero[(int64_t)layer * E + i] = 0;
-    if (origin_do) {
-        const int *Dl = Dg + (int64_t)layer * E * E;
-        long long acc = 0;
-        for (int64_t idx = threadIdx.x; idx < (int64_t)E * E; idx += blockDim.x) {
-            const int i = (int)(idx / E), j = (int)(idx % E);
-            if (i != j) {
-                const long long d = Dl[idx];
-                acc += d * d;
-            }
-        }
-        s_red[threadIdx.x] = acc;
-        __syncthreads();
-        for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-            if (threadIdx.x < o) s_red[threadIdx.x] += s_red[threadIdx.x + o];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) origin_do[layer] = s_red[0];
-    }
 }
 
-// origin_do alone (Eq. origin_do), one CTA per problem, exact in int64.
+// origin_do += sum_{i != j} D_ij^2 over kOriginRows rows of one problem (Eq.
+// origin_do), exact in int64; origin_do zero on entry.  (One CTA for a whole
+// problem, with a division per entry, took 23 us at E = 96.)
+constexpr int kOriginRows = 8;
 __global__ void __launch_bounds__(256)
 origin_do_kernel(const int *__restrict__ Dg, int E, long long *__restrict__ origin_do) {
-    __shared__ long long s_red[256];
-    const int *Dl = Dg + (int64_t)blockIdx.x * E * E;
+    __shared__ long long s_red[8];
+    const int *Dl = Dg + (int64_t)blockIdx.y * E * E;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i = blockIdx.x * kOriginRows + warp;  // a row per warp
     long long acc = 0;
-    for (int64_t idx = threadIdx.x; idx < (int64_t)E * E; idx += blockDim.x) {
-        const int i = (int)(idx / E), j = (int)(idx % E);
-        if (i != j) {
-            const long long d = Dl[idx];
+    if (i < E)
+#pragma unroll 4
+        for (int j = lane; j < E; j += 32) {
+            const long long d = j == i ? 0 : __ldg(Dl + (int64_t)i * E + j);
             acc += d * d;
         }
-    }
-    s_red[threadIdx.x] = acc;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
+    if (lane == 0) s_red[warp] = acc;
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) s_red[threadIdx.x] += s_red[threadIdx.x + o];
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        long long sum = 0;
+        for (int q = 0; q < 8; ++q) sum += s_red[q];
+        atomicAdd(reinterpret_cast<unsigned long long *>(origin_do + blockIdx.y), (unsigned long long)sum);
     }
-    if (threadIdx.x == 0) origin_do[blockIdx.x] = s_red[0];
 }
 
+// CTAs per problem and the split of a word over warps: one wave of the CTAs
+// that fit (an SM holds one with a large D in shared memory), every warp with
+// as few tokens as that allows.
+template <int R>
+void loss_generic_grid(const Problem &p, size_t smem, int P_max, int *P, int *split) {
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) == cudaSuccess)
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int warps = loss_warps<R>();
+    const int by_smem = (int)(220 * 1024 / (smem + 8 * 1024));
+    const int occ = by_smem < 1 ? 1 : by_smem > 2 ? 2 : by_smem;
+    int64_t ctas = (int64_t)sms * occ / p.L;
+    if (ctas < 1) ctas = 1;
+    int s = 1;
+    while (s < 32 && p.W * s < ctas * warps) s *= 2;
+    const int64_t need = (p.W * s + warps - 1) / warps;
+    if (ctas > need) ctas = need;
+    if (ctas > P_max) ctas = P_max;
+    *P = (int)ctas;
+    *split = s;
+}
+
+struct GenericArgs {
+    const float *logits;
+    const uint32_t *bits;
+    const int *D, *counts;
+    float coef;
+    float *dlogits;
+    double *partials;
+    int P_max;
+    int *status;
+};
+
 template <int R, bool kSmemD, int kGate>
-cudaError_t run_loss(const float *logits, const uint32_t *bits, const int *D, const Problem &p,
-                     float coef, float *dlogits, double *partials, int P, int *status,
-                     cudaStream_t s) {
+cudaError_t run_loss(const GenericArgs &a, const Problem &p, int *P, cudaStream_t s) {
     const size_t smem = sizeof(int) * ((kSmemD ? (size_t)p.E * p.E : 0) + (size_t)p.E);
     auto kern = loss_generic_kernel<R, kSmemD, kGate>;
     if (smem > 48 * 1024) {
@@ -228,28 +298,25 @@ cudaError_t run_loss(const float *logits, const uint32_t *bits, const int *D, co
                                              (int)smem);
         if (e != cudaSuccess) return e;
     }
-    dim3 grid((unsigned)P, (unsigned)p.L);
-    kern<<<grid, kLossThreads, smem, s>>>(logits, bits, D, p.T, p.E, p.W, coef, dlogits, partials,
-                                          P, status);
+    int split = 1;
+    loss_generic_grid<R>(p, smem, a.P_max, P, &split);
+    dim3 grid((unsigned)*P, (unsigned)p.L);
+    kern<<<grid, loss_warps<R>() * 32, smem, s>>>(a.logits, a.bits, a.D, a.counts, p.T, p.E, p.k, p.W,
+                                                 split, a.coef, a.dlogits, a.partials, *P, a.status);
     return cudaGetLastError();
 }
 
 template <int R>
-cudaError_t dispatch_gate(const float *logits, const uint32_t *bits, const int *D, const Problem &p,
-                          int gate, float coef, float *dlogits, double *partials, int P,
-                          int *status, cudaStream_t s) {
+cudaError_t dispatch_gate(const GenericArgs &a, const Problem &p, int gate, int *P, cudaStream_t s) {
     const bool smem_d = sizeof(int) * ((size_t)p.E * p.E + p.E) <= kSmemDLimit;
-    if (gate == 0)
-        return smem_d ? run_loss<R, true, 0>(logits, bits, D, p, coef, dlogits, partials, P, status, s)
-                      : run_loss<R, false, 0>(logits, bits, D, p, coef, dlogits, partials, P, status, s);
-    return smem_d ? run_loss<R, true, 1>(logits, bits, D, p, coef, dlogits, partials, P, status, s)
-                  : run_loss<R, false, 1>(logits, bits, D, p, coef, dlogits, partials, P, status, s);
+    if (gate == 0) return smem_d ? run_loss<R, true, 0>(a, p, P, s) : run_loss<R, false, 0>(a, p, P, s);
+    return smem_d ? run_loss<R, true, 1>(a, p, P, s) : run_loss<R, false, 1>(a, p, P, s);
 }
 
 }  // namespace
 
 int loss_blocks_per_problem(const Problem &p) {
-    int64_t blocks = (p.W + kLossWarps - 1) / kLossWarps;
+    int64_t blocks = (p.W + 7) / 8;
     int64_t cap = 1024 / p.L;
     if (cap < 1) cap = 1;
     if (blocks > cap) blocks = cap;
@@ -293,22 +360,24 @@ int max_sig_ctas_per_problem(const Problem &p) {
 cudaError_t launch_loss(const float *logits, const uint32_t *bits, const int *D, const Problem &p,
                         int gate, float d_scale, float grad_scale, float *loss,
                         long long *origin_do, float *dlogits, int *status, double *partials,
-                        cudaStream_t s, int *n_zero) {
-    const int P = loss_blocks_per_problem(p);
+                        cudaStream_t s, const int *counts, int *n_zero) {
     const double norm = 1.0 / ((double)p.T * (double)p.T * (double)p.k);
-    const float coef = (float)((double)grad_scale * (double)d_scale * norm);
+    const GenericArgs a = {logits, bits, D, counts, (float)((double)grad_scale * (double)d_scale * norm),
+                           dlogits, partials, ws_layout(p, false).max_parts, status};
     const int r = (p.E + 31) / 32;
+    int P = 1;
     cudaError_t e;
-    if (r <= 1) e = dispatch_gate<1>(logits, bits, D, p, gate, coef, dlogits, partials, P, status, s);
-    else if (r <= 2) e = dispatch_gate<2>(logits, bits, D, p, gate, coef, dlogits, partials, P, status, s);
-    else if (r <= 4) e = dispatch_gate<4>(logits, bits, D, p, gate, coef, dlogits, partials, P, status, s);
-    else if (r <= 8) e = dispatch_gate<8>(logits, bits, D, p, gate, coef, dlogits, partials, P, status, s);
-    else if (r <= 16) e = dispatch_gate<16>(logits, bits, D, p, gate, coef, dlogits, partials, P, status, s);
-    else e = dispatch_gate<32>(logits, bits, D, p, gate, coef, dlogits, partials, P, status, s);
+    if (r <= 1) e = dispatch_gate<1>(a, p, gate, &P, s);
+    else if (r <= 2) e = dispatch_gate<2>(a, p, gate, &P, s);
+    else if (r <= 4) e = dispatch_gate<4>(a, p, gate, &P, s);
+    else if (r <= 8) e = dispatch_gate<8>(a, p, gate, &P, s);
+    else if (r <= 16) e = dispatch_gate<16>(a, p, gate, &P, s);
+    else e = dispatch_gate<32>(a, p, gate, &P, s);
     if (e != cudaSuccess) return e;
-    loss_finalize_kernel<<<p.L, 256, 0, s>>>(partials, P, D, p.E, (double)d_scale * norm, loss,
-                                             origin_do, n_zero);
-    return cudaGetLastError();
+    loss_finalize_kernel<<<p.L, 256, 0, s>>>(partials, P, p.E, (double)d_scale * norm, loss, n_zero);
+    e = cudaGetLastError();
+    if (e == cudaSuccess && origin_do) e = launch_origin_do(D, p, origin_do, s);
+    return e;
 }
 
 // Variance of the E (E - 1) off-diagonal distances of a local window from
@@ -331,7 +400,10 @@ cudaError_t launch_offdiag_variance(const long long *origin_do, const Problem &p
 }
 
 cudaError_t launch_origin_do(const int *D, const Problem &p, long long *origin_do, cudaStream_t s) {
-    origin_do_kernel<<<p.L, 256, 0, s>>>(D, p.E, origin_do);
+    cudaError_t e = cudaMemsetAsync(origin_do, 0, sizeof(long long) * (size_t)p.L, s);
+    if (e != cudaSuccess) return e;
+    origin_do_kernel<<<dim3((unsigned)((p.E + kOriginRows - 1) / kOriginRows), (unsigned)p.L), 256, 0, s>>>(
+        D, p.E, origin_do);
     return cudaGetLastError();
 }
 
