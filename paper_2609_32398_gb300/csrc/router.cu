@@ -20,14 +20,17 @@
 //   warps 2-5 epilogue, one TMEM lane quarter each (the same 32 rows of both
 //            tiles): the logits go TMEM -> registers -> a swizzled shared-memory
 //            tile (the signature kernel's layout), out to HBM by TMA stores, and
-//            the signature kernel's per-token selection and signature words run
-//            on that tile.  The co-occurrence counts go into a shared triangle
+//            the selection by sorting networks (select_net, which only reads
+//            the tile; half the instructions of the argmax rounds, on the four
+//            warps that end the kernel) and the signature words run on that
+//            tile.  The co-occurrence counts go into a shared triangle
 //            of 16-bit counters (two per word: the CTA's range is below 65536
 //            tokens), written out unpacked at the end; for longer ranges they
 //            go straight to the CTA's triangle in global memory as L2
 //            reductions.
 
 #include "sig_fast.cuh"
+#include "topk_net.cuh"
 
 namespace dol {
 namespace {
@@ -65,6 +68,32 @@ struct RouterArgs {
     ZeroSpans zero;
     int *status;
 };
+
+// The signature words of the warp's 32 tokens (lane = token): a bit per chosen
+// expert, turned into one word per expert by 32x32 bit transposes; lane c
+// stores the word of expert 32 r + c at words[(32 r + c) W].  With kCount,
+// cnt[r] accumulates the word's population count.
+template <int E, int K, bool kCount>
+__device__ __forceinline__ void emit_words(const int (&sel)[K], bool valid, int lane,
+                                           uint32_t *words, int64_t W, uint32_t (&cnt)[E / 32]) {
+    constexpr int R = E / 32;
+    uint32_t m[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) m[r] = 0u;
+#pragma unroll
+    for (int qk = 0; qk < K; ++qk) {
+        const uint32_t bit = 1u << (sel[qk] & 31);
+        const int rq = sel[qk] >> 5;
+#pragma unroll
+        for (int r = 0; r < R; ++r) m[r] |= (rq == r) ? bit : 0u;
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const uint32_t word = transpose32_bits(valid ? m[r] : 0u, lane);
+        words[(int64_t)(32 * r + lane) * W] = word;
+        if (kCount) cnt[r] += __popc(word);
+    }
+}
 
 // Words of the next tile of a range with r words left: pairs of MMA tiles
 // (eight words) that share each slice of W, the remainder last.
@@ -256,28 +285,16 @@ router_sig_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constan
                 }
                 const int64_t t = (int64_t)row0 + lane;
                 const bool valid = t < a.T;
-                int sel[K];
-                float val[K];
-                select_topk<kRE, K, true>(tp, lane, sel, val);
+                int sel[K];  // ascending
+                select_net<kRE / 32, K>(tp, lane, valid, sel);
                 if (a.idx && valid) store_idx<K>(a.idx + ((int64_t)layer * a.T + t) * K, sel);
                 if (valid) {  // c_ab += 1 for the pairs a < b, 16-bit halves of shared words
-                    int so[K];
 #pragma unroll
-                    for (int q = 0; q < K; ++q) so[q] = sel[q];
+                    for (int q2 = 1; q2 < K; ++q2) {
+                        const int col = s_coloff[sel[q2]];
 #pragma unroll
-                    for (int i2 = 1; i2 < K; ++i2)
-#pragma unroll
-                        for (int j2 = i2; j2 > 0; --j2) {
-                            const int lo = min(so[j2 - 1], so[j2]), hi = max(so[j2 - 1], so[j2]);
-                            so[j2 - 1] = lo;
-                            so[j2] = hi;
-                        }
-#pragma unroll
-                    for (int q1 = 0; q1 < K - 1; ++q1) {
-                        const int row = 4 * so[q1];
-#pragma unroll
-                        for (int q2 = q1 + 1; q2 < K; ++q2) {
-                            const int wi = row + s_coloff[so[q2]];
+                        for (int q1 = 0; q1 < q2; ++q1) {
+                            const int wi = col + 4 * sel[q1];
                             if (a.packed) atomicAdd(&s_tri[wi >> 1], 1u << (16 * (wi & 1)));
                             else atomicAdd(&tri[wi], 1u);
                         }

@@ -35,10 +35,10 @@
 
 #include "dol_internal.cuh"
 #include "tma.cuh"
+#include "topk_net.cuh"
 
 namespace dol {
 
-constexpr int kSelBoxBytes = 32 * 128;  // 32 rows x 32 fp32
 constexpr int kSelMaxSlots = 16;
 // Most teams (pairs of consumer warps) and block size for lists of KP values:
 // the launch bound keeps 72 registers a thread for KP <= 8, so that the
@@ -101,171 +101,6 @@ struct SelArgs {
 };
 
 namespace {
-
-// Transpose a 32x32 bit matrix held one row per lane (bit c of lane t is
-// element (t, c)); on return lane c holds column c (bit t = element (t, c)).
-// Each step exchanges j x j blocks: a rotation of the partner's word by j (up
-// or down, by lane) and one bit select.
-__device__ __forceinline__ uint32_t transpose32_bits(uint32_t x, int lane) {
-    const uint32_t lo_mask[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
-#pragma unroll
-    for (int s = 0; s < 5; ++s) {
-        const int j = 16 >> s;
-        const uint32_t p = __shfl_xor_sync(kFull, x, j);
-        const uint32_t keep = (lane & j) ? ~lo_mask[s] : lo_mask[s];
-        const uint32_t r = __funnelshift_l(p, p, (lane & j) ? 32 - j : j);
-        x = (x & keep) | (r & ~keep);
-    }
-    return x;
-}
-
-__device__ __forceinline__ uint32_t h2max(uint32_t a, uint32_t b) {
-    uint32_t d;
-    asm("max.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-    return d;
-}
-__device__ __forceinline__ uint32_t h2min(uint32_t a, uint32_t b) {
-    uint32_t d;
-    asm("min.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-    return d;
-}
-// two values rounded towards zero to fp16: lo in the low half
-__device__ __forceinline__ uint32_t pack_rz(float lo, float hi) {
-    uint32_t d;
-    asm("cvt.rz.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
-    return d;
-}
-
-// v[i] >= v[j] in both halves
-__device__ __forceinline__ void ce(uint32_t &a, uint32_t &b) {
-    const uint32_t hi = h2max(a, b), lo = h2min(a, b);
-    a = hi;
-    b = lo;
-}
-
-// Batcher's odd-even merge sort of positions LO .. LO + N - 1; cx(i, j) puts
-// the larger of two positions first.
-template <int LO, int N, int R, class Cx>
-__device__ __forceinline__ void net_merge(const Cx &cx) {
-    if constexpr (2 * R < N) {
-        net_merge<LO, N, 2 * R>(cx);
-        net_merge<LO + R, N, 2 * R>(cx);
-#pragma unroll
-        for (int i = LO + R; i + R < LO + N; i += 2 * R) cx(i, i + R);
-    } else {
-        cx(LO, LO + R);
-    }
-}
-template <int LO, int N, class Cx>
-__device__ __forceinline__ void net_sort(const Cx &cx) {
-    if constexpr (N > 1) {
-        net_sort<LO, N / 2>(cx);
-        net_sort<LO + N / 2, N / 2>(cx);
-        net_merge<LO, N, 1>(cx);
-    }
-}
-
-// N packed pairs sorted in both halves, largest first.
-template <int N>
-__device__ __forceinline__ void sort_desc(uint32_t (&v)[N]) {
-    net_sort<0, N>([&](int i, int j) { ce(v[i], v[j]); });
-}
-
-// a = the N largest of two lists a and b sorted largest first, sorted again:
-// max(a_i, b_(N-1-i)) are those N as a bitonic sequence.
-template <int N>
-__device__ __forceinline__ void merge_top(uint32_t (&a)[N], const uint32_t (&b)[N]) {
-#pragma unroll
-    for (int i = 0; i < N; ++i) a[i] = h2max(a[i], b[N - 1 - i]);
-#pragma unroll
-    for (int h = N / 2; h >= 1; h >>= 1)
-#pragma unroll
-        for (int i = 0; i < N; ++i)
-            if ((i & h) == 0) ce(a[i], a[i + h]);
-}
-
-// Byte address of float4 chunk c of box b of this lane's row in a swizzled tile.
-__device__ __forceinline__ unsigned char *sel_chunk(unsigned char *tile, int b, int c, int lane) {
-    return tile + b * kSelBoxBytes + lane * 128 + ((c ^ (lane & 7)) << 4);
-}
-__device__ __forceinline__ float sel_value(unsigned char *tile, int e, int lane) {
-    return reinterpret_cast<const float *>(sel_chunk(tile, e >> 5, (e & 31) >> 2, lane))[e & 3];
-}
-
-// The KP largest values of boxes [b0, b1) of this lane's row at fp16 precision,
-// largest first (the same list in both halves).
-template <int KP>
-__device__ __forceinline__ void topk_lists(unsigned char *tile, int b0, int b1, int lane,
-                                           uint32_t (&top)[KP]) {
-    // one copy of the code for every box: with two boxes unrolled the warps,
-    // each at another place of a longer kernel, waited for instructions
-    // (2.2 cycles per issue against 0.4)
-#pragma unroll 1
-    for (int b = b0; b < b1; ++b) {
-        constexpr int G = 16 / KP;  // packed groups of KP pairs in 32 experts
-        uint32_t h[G][KP];
-#pragma unroll
-        for (int g = 0; g < G; ++g)
-#pragma unroll
-            for (int c = 0; c < KP / 4; ++c) {
-                const float4 x = *reinterpret_cast<const float4 *>(
-                    sel_chunk(tile, b, (2 * g) * (KP / 4) + c, lane));
-                const float4 y = *reinterpret_cast<const float4 *>(
-                    sel_chunk(tile, b, (2 * g + 1) * (KP / 4) + c, lane));
-                h[g][4 * c] = pack_rz(x.x, y.x);
-                h[g][4 * c + 1] = pack_rz(x.y, y.y);
-                h[g][4 * c + 2] = pack_rz(x.z, y.z);
-                h[g][4 * c + 3] = pack_rz(x.w, y.w);
-            }
-#pragma unroll
-        for (int g = 0; g < G; ++g) sort_desc<KP>(h[g]);
-#pragma unroll
-        for (int s = 1; s < G; s <<= 1)
-#pragma unroll
-            for (int g = 0; g + s < G; g += 2 * s) merge_top<KP>(h[g], h[g + s]);
-        if (b == b0) {
-#pragma unroll
-            for (int i = 0; i < KP; ++i) top[i] = h[0][i];
-        } else {
-            merge_top<KP>(top, h[0]);
-        }
-    }
-    // the halves' lists against each other: the same list in both
-    uint32_t other[KP];
-#pragma unroll
-    for (int i = 0; i < KP; ++i) other[i] = __byte_perm(top[i], 0u, 0x1032);
-    merge_top<KP>(top, other);
-}
-
-// The smallest fp32 that rounds (towards zero) to the k-th largest value of
-// the sorted list top, or of top and other together.
-template <int KP>
-__device__ __forceinline__ float topk_bound(uint32_t (&top)[KP], const uint32_t *other, int k) {
-    uint32_t kth;
-    if (other && k == KP) {  // the smallest of the KP largest of both
-        kth = h2max(top[0], other[(KP - 1) * 32]);
-#pragma unroll
-        for (int i = 1; i < KP; ++i) kth = h2min(kth, h2max(top[i], other[(KP - 1 - i) * 32]));
-    } else {
-        if (other) {
-            uint32_t o[KP];
-#pragma unroll
-            for (int i = 0; i < KP; ++i) o[i] = other[i * 32];
-            merge_top<KP>(top, o);
-        }
-        kth = top[0];
-#pragma unroll
-        for (int i = 1; i < KP; ++i) kth = (i < k) ? top[i] : kth;
-    }
-    kth &= 0xFFFFu;
-    if (kth > 0u && kth < 0x8000u) return __half2float(__ushort_as_half((unsigned short)kth));
-    // zero or negative: the fp32 values that round to it reach down to, but
-    // not as far as, the next fp16 below
-    uint32_t mag = kth & 0x7FFFu;
-    if (mag > 0x7BFFu) mag = 0x7BFFu;
-    const float next = __half2float(__ushort_as_half((unsigned short)(mag + 1u)));
-    return __uint_as_float((__float_as_uint(next) - 1u) | 0x80000000u);
-}
 
 // Barrier of the `n` threads of one tile's warps; the AND of ok over them.
 __device__ __forceinline__ bool tile_sync_and(int id, int n, bool ok) {

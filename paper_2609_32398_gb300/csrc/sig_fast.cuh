@@ -15,8 +15,7 @@
 //      memory, and the group maximum is recomputed.
 // Each lane sets its token's bit in the words of its K chosen experts with
 // shared-memory atomic ORs into a per-warp scratch of E words, from which
-// lane c stores the words of experts c, c + 32, ... (the router kernel, whose
-// shared memory is full, builds the same words by 32x32 bit transposes).
+// lane c stores the words of experts c, c + 32, ...
 // The k selected indices of every token are also written (one byte each) for
 // the loss kernel, and the CTAs zero the accumulators of the next kernels.
 // The routing instantiations (kRoute) also write, per token, the chosen
@@ -54,20 +53,6 @@ struct SigCfg {
                                     (size_t)kConsumers * E * 4;
 };
 
-
-// Transpose a 32x32 bit matrix held one row per lane (bit c of lane t is
-// element (t, c)); on return lane c holds column c (bit t = element (t, c)).
-__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
-    const uint32_t lo_mask[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
-#pragma unroll
-    for (int s = 0; s < 5; ++s) {
-        const int j = 16 >> s;
-        const uint32_t lo = lo_mask[s];
-        const uint32_t p = __shfl_xor_sync(kFull, x, j);
-        x = (lane & j) ? ((x & ~lo) | ((p >> j) & lo)) : ((x & lo) | ((p << j) & ~lo));
-    }
-    return x;
-}
 
 // Byte address of float4 chunk e4 of this lane's row inside a swizzled tile.
 __device__ __forceinline__ unsigned char *chunk_ptr(unsigned char *tile, int e4, int lane) {
@@ -130,15 +115,10 @@ __device__ __forceinline__ void store_route(const RouteOut &r, int64_t off, cons
 // (lowest index among equal values), overwritten with -inf in the tile, and
 // the group maximum recomputed.  sel: the chosen experts in selection order;
 // val: their logits.
-// kMask: chosen experts are excluded through a per-lane bit mask instead of
-// -inf writes, so the tile is only read (it may be in flight to HBM meanwhile).
-template <int E, int K, bool kMask = false>
+template <int E, int K>
 __device__ __forceinline__ void select_topk(unsigned char *tp, int lane, int (&sel)[K],
                                             float (&val)[K]) {
     constexpr int GS = SigCfg<E>::GS, NG = SigCfg<E>::NG, GS4 = GS / 4;
-    uint32_t chosen[E / 32];
-#pragma unroll
-    for (int r = 0; r < E / 32; ++r) chosen[r] = 0u;
     float g[NG];
 #pragma unroll
     for (int gi = 0; gi < NG; ++gi) {
@@ -180,14 +160,6 @@ __device__ __forceinline__ void select_topk(unsigned char *tp, int lane, int (&s
             x[4 * c + 2] = v.z;
             x[4 * c + 3] = v.w;
         }
-        if (kMask) {  // the experts of this group chosen before
-            uint32_t word = 0u;
-#pragma unroll
-            for (int r = 0; r < E / 32; ++r) word = ((bi * GS) >> 5) == r ? chosen[r] : word;
-            const uint32_t gm = (word >> ((bi * GS) & 31)) & ((1u << GS) - 1u);
-#pragma unroll
-            for (int j = 0; j < GS; ++j) x[j] = ((gm >> j) & 1u) ? -INFINITY : x[j];
-        }
         int p = GS - 1;
 #pragma unroll
         for (int j = GS - 1; j >= 0; --j)
@@ -196,12 +168,7 @@ __device__ __forceinline__ void select_topk(unsigned char *tp, int lane, int (&s
 #pragma unroll
         for (int j = 0; j < GS; ++j) m2 = fmaxf(m2, j == p ? -INFINITY : x[j]);
         const int e = bi * GS + p;
-        if (kMask) {
-#pragma unroll
-            for (int r = 0; r < E / 32; ++r) chosen[r] |= (e >> 5) == r ? 1u << (e & 31) : 0u;
-        } else {
-            reinterpret_cast<float *>(chunk_ptr(tp, e >> 2, lane))[e & 3] = -INFINITY;
-        }
+        reinterpret_cast<float *>(chunk_ptr(tp, e >> 2, lane))[e & 3] = -INFINITY;
 #pragma unroll
         for (int gi = 0; gi < NG; ++gi) g[gi] = (gi == bi) ? m2 : g[gi];
         sel[qk] = e;
@@ -245,32 +212,6 @@ __device__ __forceinline__ void cooc_add(uint32_t *s_cooc, const int *s_coloff, 
         uint32_t *col = s_cooc + s_coloff[so[q2]];
 #pragma unroll
         for (int q1 = 0; q1 < q2; ++q1) atomicAdd(col + 4 * so[q1], 1u);
-    }
-}
-
-// The signature words of the warp's 32 tokens (lane = token): a bit per chosen
-// expert, turned into one word per expert by 32x32 bit transposes; lane c
-// stores the word of expert 32 r + c at words[(32 r + c) W].  With kCount,
-// cnt[r] accumulates the word's population count.
-template <int E, int K, bool kCount>
-__device__ __forceinline__ void emit_words(const int (&sel)[K], bool valid, int lane,
-                                           uint32_t *words, int64_t W, uint32_t (&cnt)[E / 32]) {
-    constexpr int R = E / 32;
-    uint32_t m[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) m[r] = 0u;
-#pragma unroll
-    for (int qk = 0; qk < K; ++qk) {
-        const uint32_t bit = 1u << (sel[qk] & 31);
-        const int rq = sel[qk] >> 5;
-#pragma unroll
-        for (int r = 0; r < R; ++r) m[r] |= (rq == r) ? bit : 0u;
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const uint32_t word = transpose32(valid ? m[r] : 0u, lane);
-        words[(int64_t)(32 * r + lane) * W] = word;
-        if (kCount) cnt[r] += __popc(word);
     }
 }
 
