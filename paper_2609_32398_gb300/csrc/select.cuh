@@ -415,6 +415,7 @@ select_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ 
         const int threads = 32 * split, bar_id = 1 + team;
         const int bm = (nb + 1) / 2;  // boxes of the first warp
         const int b0 = part == 0 ? 0 : bm, b1 = (part == 0 && split > 1) ? bm : nb;
+        const uint32_t in_last = (E & 31) ? kFull << (32 - (E & 31)) : kFull;  // columns of the last box below E
         uint32_t *list = reinterpret_cast<uint32_t *>(smem + a.lay.off_list) + team * 2 * KP * 32 + lane;
         uint32_t *masks = reinterpret_cast<uint32_t *>(smem + a.lay.off_mask) + team * (nb + 2) * 32 + lane;
         for (int q = team, s = team, round = 0; q < n; q += teams, s += teams) {
@@ -460,7 +461,7 @@ select_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ 
                     below = __funnelshift_l(__float_as_uint(v.z - bound), below, 1);
                     below = __funnelshift_l(__float_as_uint(v.w - bound), below, 1);
                 }
-                const uint32_t cand = valid ? ~below : 0u;
+                const uint32_t cand = valid ? ~below & (b == nb - 1 ? in_last : kFull) : 0u;
                 cnt += __popc(cand);
                 masks[b * 32] = cand;
             }

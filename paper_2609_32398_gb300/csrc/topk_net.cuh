@@ -172,6 +172,9 @@ __device__ __forceinline__ float topk_bound(uint32_t (&top)[KP], const uint32_t 
     }
     kth &= 0xFFFFu;
     if (kth > 0u && kth < 0x8000u) return __half2float(__ushort_as_half((unsigned short)kth));
+    // minus infinity is the image of nothing else (-inf - -inf is a NaN without
+    // a sign bit: not below)
+    if (kth == 0xFC00u) return -INFINITY;
     // zero or negative: the fp32 values that round to it reach down to, but
     // not as far as, the next fp16 below
     uint32_t mag = kth & 0x7FFFu;

@@ -1,0 +1,171 @@
+"""The selection kernel (topk_net.cuh, select.cuh), the co-occurrence reduction
+and the loss kernels (loss_mma.cuh, loss.cu) at the sizes where their tiles,
+paddings and splits end, against the CPU oracle.
+
+Signatures, counts, D, origin_do and the routing integers are exact.
+
+Loss and dlogits, per entry.  With p the gate's weights, w = dL/dp (fp64, from
+the oracle) and M_t = sum_i p_it |w_it|, the kernels compute
+dz_it = p_it (1 - s_it) (w_it - A_t) (softmax: p_it (w_it - A_t)), A_t = sum_i
+p_it w_it.  The sums over E columns are fp32 (E u each, u = 2^-24); s comes from
+one ex2.approx (2 ulp) of a product rounded at |z| <= 8 (12 u) and one rcp.approx
+(1 ulp), so s, the sums and their quotient are within (E + 64) u; the integers
+behind w are exact below 2^24 and rounded once above.  So
+  |dz - ref| <= 2 (E + 64) u p (1 - s) (|w| + M_t),  |loss - ref| <= 2 (E + 64) u sum_t M_t,
+the factor 2 for the two factors of the product.  u p_max max|w| is added for
+results rounded near zero.
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2609_32398_gb300 import workloads
+from test_routed_split_gpu import route_bound
+
+pytestmark = pytest.mark.gpu
+
+U = 2.0 ** -24
+
+
+@pytest.fixture(scope="module")
+def dl():
+    import paper_2609_32398_gb300.doloss as m
+
+    m.lib()
+    return m
+
+
+def check_loss(z, f, D, k, gate, loss, dz, d_scale=1.0, extra=0.0, extra_bound=0.0):
+    T, E = z.shape
+    p = oracle.gate(z, gate)
+    w = oracle.dloss_dp(D, f, T, k, d_scale)
+    M = (p * np.abs(w)).sum(1, keepdims=True)
+    ref = oracle.loss(D, oracle.direction(z, f, gate), T, k, d_scale)
+    tol = 2.0 * (E + 64) * U
+    assert abs(loss - ref) <= tol * M.sum() + U * abs(ref), ("loss", loss, ref)
+    if dz is None:
+        return
+    oms = 1.0 if gate == workloads.GATE_SOFTMAX else 1.0 / (1.0 + np.exp(z.astype(np.float64)))
+    bound = tol * p * oms * (np.abs(w) + M) + U * p.max() * np.abs(w).max()
+    err = np.abs(dz.double().cpu().numpy() - oracle.gate_backward(z, w, gate) - extra)
+    bound = bound + extra_bound
+    assert (err <= bound).all(), ("dlogits", float((err / bound).max()))
+
+
+# four experts, a width that is no multiple of 32, every number of 32-expert
+# boxes, lists of 4, 8 and 16, one token, ragged and whole tiles, ties
+@pytest.mark.parametrize("T,E,k,L,ties", [
+    (1, 4, 1, 1, False), (33, 4, 4, 3, True), (31, 12, 3, 1, True), (257, 36, 9, 2, True),
+    (500, 64, 5, 1, False), (1000, 96, 6, 2, True), (97, 100, 16, 1, True), (64, 128, 16, 1, True),
+    (129, 160, 2, 1, True), (700, 200, 7, 1, False), (4801, 256, 8, 1, True), (333, 256, 16, 2, True),
+    (65, 384, 12, 1, True), (2049, 512, 10, 1, True), (32, 512, 16, 2, False)])
+def test_selection(dl, T, E, k, L, ties):
+    z = workloads.random_logits(T, E, L=L, seed=31 * T + E + k, ties=ties)
+    z[0, 0, : min(E, k + 1)] = -torch.inf            # ties of the lowest value
+    if E >= 8:
+        z[L - 1, T - 1, E // 2:] = torch.finfo(torch.float32).min
+    zc = z.cuda()
+    bits, counts = dl.signatures(zc, k)
+    finite = z.clone()
+    finite[0, 0] = torch.arange(E, dtype=torch.float32) % 3    # its combine weights are defined
+    r = dl.routing(finite.cuda(), k, workloads.GATE_SOFTMAX)
+    assert dl.device_status(r.workspace) == 0
+    for l in range(L):
+        f = oracle.select(z[l].numpy(), k)
+        assert np.array_equal(bits[l].cpu().numpy().view(np.uint32), oracle.pack(f))
+        assert np.array_equal(counts[l].cpu().numpy(), oracle.counts(f))
+        ids, comb = oracle.route(finite[l].numpy(), k, workloads.GATE_SOFTMAX)
+        assert np.array_equal(r.expert_ids[l].cpu().numpy(), ids)
+        # k terms summed, exponentials of 2 ulp: (k + 12) u, doubled
+        assert np.abs(r.combine[l].double().cpu().numpy() - comb).max() <= 2 * (k + 12) * U
+        offsets, rows, pos = oracle.dispatch(ids, E)
+        assert np.array_equal(r.offsets[l].cpu().numpy(), offsets)
+        assert np.array_equal(r.rows[l].cpu().numpy(), rows)
+        assert np.array_equal(r.pos[l].cpu().numpy(), pos)
+
+
+# one to four boxes of the tensor-core kernel, padded and whole; tiles of 128
+# tokens and their remainders; both gates; the marker diagonal ((E - 1) T >=
+# 2^23); counted widths above 128 and the generic kernel (k > 64, E > 256)
+@pytest.mark.parametrize("T,E,k,L,gate", [
+    (1, 4, 1, 1, 0), (127, 12, 3, 2, 1), (129, 32, 16, 1, 0), (1300, 36, 4, 1, 1), (128, 64, 5, 3, 0),
+    (641, 68, 7, 1, 0), (255, 96, 6, 2, 1), (20011, 100, 8, 1, 0), (385, 128, 10, 2, 1),
+    (2000, 128, 3, 1, 0), (66053, 128, 5, 1, 0), (84737, 100, 8, 1, 1),
+    (300, 132, 8, 1, 0), (777, 160, 16, 2, 1), (1000, 252, 3, 1, 0),
+    (130, 100, 70, 2, 1), (99, 300, 5, 1, 0), (4099, 320, 9, 2, 1), (33, 1000, 12, 1, 0)])
+def test_step(dl, T, E, k, L, gate):
+    z = workloads.random_logits(T, E, L=L, seed=T + 7 * E + k)
+    zc = z.cuda()
+    out = dl.forward_backward(zc, k, gate)
+    fwd = dl.forward_backward(zc, k, gate, with_grad=False)
+    again = dl.forward_backward(zc, k, gate, out=dl.Buffers(L, T, E, k))
+    torch.cuda.synchronize()
+    assert dl.device_status(out.workspace) == 0 and dl.device_status(fwd.workspace) == 0
+    assert torch.equal(out.dlogits, again.dlogits) and torch.equal(out.loss, again.loss)
+    for l in range(L):
+        zl = z[l].numpy()
+        f = oracle.select(zl, k)
+        D = oracle.hamming(f)
+        for o in (out, fwd):
+            assert np.array_equal(o.bits[l].cpu().numpy().view(np.uint32), oracle.pack(f))
+            assert np.array_equal(o.counts[l].cpu().numpy(), oracle.counts(f))
+            assert np.array_equal(o.D[l].cpu().numpy(), D)
+            assert int(o.origin_do[l]) == oracle.origin_do(D)
+        check_loss(zl, f, D, k, gate, float(out.loss[l]), out.dlogits[l])
+        check_loss(zl, f, D, k, gate, float(fwd.loss[l]), None)
+
+
+# a given matrix: its image (the first problem), and one that no image holds (an
+# entry of 2^22, or a non-zero diagonal), gathered from D in the same launch
+@pytest.mark.parametrize("T,E,k,gate,fault", [
+    (200, 36, 5, 0, "large"), (515, 128, 8, 1, "diagonal"), (260, 96, 3, 0, "diagonal"),
+    (129, 64, 8, 1, "large")])
+def test_given_matrix(dl, T, E, k, gate, fault):
+    z = workloads.random_logits(T, E, L=2, seed=T + E)
+    f = [oracle.select(z[l].numpy(), k) for l in range(2)]
+    D = np.stack([3 * oracle.hamming(x) for x in f])
+    if fault == "large":
+        D[1, 1, 3] = D[1, 3, 1] = 1 << 22
+    else:
+        D[1, 2, 2] = 5
+    bits = torch.from_numpy(np.stack([oracle.pack(x) for x in f]).view(np.int32)).cuda()
+    loss, origin, dz = dl.loss_fwd_bwd(z.cuda(), bits, torch.from_numpy(D).cuda(), k, gate, d_scale=0.5)
+    for l in range(2):
+        off = D[l].astype(np.int64) ** 2
+        assert int(origin[l]) == int(off.sum() - np.trace(off))
+        check_loss(z[l].numpy(), f[l], D[l], k, gate, float(loss[l]), dz[l], d_scale=0.5)
+
+
+# the routing gradient: the choices of a token split over four warps (k = 2: two
+# of them idle), with the marker diagonal and without
+@pytest.mark.parametrize("T,k", [(1, 8), (129, 2), (500, 4), (66053, 8)])
+def test_routing_gradient(dl, T, k):
+    E = 128
+    z = workloads.random_logits(T, E, seed=T + k)
+    g = 1e-3 * torch.randn(1, T, k, generator=torch.Generator().manual_seed(T))
+    out, r = dl.routed_forward(z.cuda(), k)
+    dl.routed_backward(z.cuda(), r.expert_ids, g.cuda(), k, out=out)
+    torch.cuda.synchronize()
+    assert dl.device_status(out.workspace) == 0
+    zl, gl = z[0].numpy(), g[0].numpy()
+    f = oracle.select(zl, k)
+    ids, _ = oracle.route(zl, k)
+    check_loss(zl, f, oracle.hamming(f), k, 0, float(out.loss[0]), out.dlogits[0],
+               extra=oracle.route_backward(zl, ids, gl), extra_bound=route_bound(zl, ids, gl, 0))
+
+
+# the narrow workspace layout: E = 256 in the library's fixed 16 MiB array where
+# the layout with counts does not fit any more
+@pytest.mark.parametrize("T", [1 << 16, 500000])
+def test_static_scratch_narrow_layout(dl, T):
+    E, k = 256, 8
+    z = workloads.random_logits(T, E, seed=T, device="cuda")
+    out, ref = dl.Buffers(1, T, E, k), dl.Buffers(1, T, E, k)
+    dl.forward_backward_static(z, k, out)
+    dl.forward_backward(z, k, out=ref)
+    torch.cuda.synchronize()
+    for a, b in ((out.bits, ref.bits), (out.counts, ref.counts), (out.D, ref.D), (out.origin_do, ref.origin_do)):
+        assert torch.equal(a, b)
+    assert float(out.loss) == pytest.approx(float(ref.loss), rel=1e-5)
+    assert (out.dlogits - ref.dlogits).abs().max() <= 1e-4 * ref.dlogits.abs().max()
