@@ -1,4 +1,6 @@
-// Step 3, fast path (E in {32, 64, 128, 256}, k in {1, 2, 4, 8}): the
+// Step 3 for k in {1, 2, 4, 8} where the tensor-core kernel (loss_mma.cuh) does
+// not apply: E = 256, and E in {32, 64, 128} from T = 2^22 on or without room for
+// its image of D'.  The
 // surrogate DO-loss and its gradient (Sec. 3.1.3, Eq. do_loss; Eq. global_do
 // scaling).
 //
@@ -27,13 +29,17 @@
 // last CTA of each problem adds the CTA partials in index order.
 //
 // At E = 256 an int32 D (256 KB) does not fit in shared memory: D is kept
-// there as a 16-bit low plane and an 8-bit high plane (192 KB; exact for the
-// matrix of the same tokens, whose entries are at most T < 2^24), with zeros
-// on the diagonal, and the -R_i of the k chosen experts are added to their
-// sums after the gather (R from the counts).  A row chunk of 4 entries is one
-// 8-byte and one 4-byte load; the low halves are summed per entry and the
-// high bytes in pairs of 16-bit fields, joined after the k rows.  One CTA of
-// 512 threads per SM.
+// there as a plane of 16-bit fields and an 8-bit plane (192 KB), with zeros on
+// the diagonal, and the -R_i of the k chosen experts are taken off their sums
+// after the gather (R from the counts).  The entries are at most T, so for
+// T < 2^21 the fields hold 13 bits and k <= 8 of them are added in place, two
+// to a word; up to 2^24 they hold 16 bits and are taken apart first.  A row
+// chunk of 4 entries is one 8-byte and one 4-byte load.  One CTA of 768 threads
+// per SM.  Bound by shared-memory loads (6 KB a token, 60% of the pipe) and the
+// latency around them: the logits two token groups ahead are requested into L2,
+// without which a warp waited longest for its own next rows.  T = 2^20, k = 8:
+// 515 us a layer against 591 us with 512 threads, without the request and with
+// 16-bit fields alone.
 #include <climits>
 
 #include "dol_internal.cuh"
@@ -44,7 +50,7 @@ namespace {
 
 constexpr int kLossFastThreads = 256;
 // E = 256: one CTA per SM (the planes of D take 192 KB), with more warps
-constexpr int kLossPlaneThreads = 512;
+constexpr int kLossPlaneThreads = 768;
 template <int E>
 constexpr int loss_fast_threads() { return E == 256 ? kLossPlaneThreads : kLossFastThreads; }
 template <int E>
@@ -110,13 +116,15 @@ struct LossArgs {
     int *status_out;  // may be null: the last CTA ORs the status word into it
 };
 
-template <int E, int K, int kGate, bool kRFromCounts>
+// kNarrow (E = 256): every entry of D is below 2^21 (at most T, T < 2^21).
+template <int E, int K, int kGate, bool kRFromCounts, bool kNarrow>
 __global__ void __launch_bounds__(loss_fast_threads<E>(), E == 256 ? 1 : 3)
 loss_fast_kernel(const LossArgs a) {
     constexpr int G = E / 16;    // lanes per token
     constexpr int TPW = 32 / G;  // tokens per warp pass
     constexpr int Q = E / 4;     // expert stride between a lane's chunks
     constexpr bool kPlanes = E == 256;
+    constexpr int kLoBits = kNarrow ? 13 : 16;  // of an entry, in the low plane
     constexpr int kWarps = loss_fast_threads<E>() / 32;
     static_assert(!kPlanes || kRFromCounts, "the planes hold the matrix of the same tokens");
     extern __shared__ __align__(128) int sD[];  // [E][E], or the two planes
@@ -125,7 +133,8 @@ loss_fast_kernel(const LossArgs a) {
     __shared__ __align__(8) uint64_t bar;
     __shared__ double s_part[kWarps];
     __shared__ long long s_o[kWarps];
-    __shared__ long long s_r[E];
+    __shared__ long long s_r[kPlanes ? 1 : E];
+    __shared__ __align__(16) int s_rp[kPlanes ? E : 4];  // R (planes)
     __shared__ int s_last;
 
     const int layer = blockIdx.y;
@@ -174,14 +183,15 @@ loss_fast_kernel(const LossArgs a) {
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 if (j0 + u == i) x[u] = 0;
-                bad |= (unsigned)x[u] >= (1u << 24);
+                bad |= (unsigned)x[u] >= (1u << (kLoBits + 8));
             }
+            constexpr uint32_t kLoMask = (1u << kLoBits) - 1u;
             *reinterpret_cast<uint2 *>(sLo + e0) =
-                make_uint2(((uint32_t)x[0] & 0xFFFFu) | ((uint32_t)x[1] << 16),
-                           ((uint32_t)x[2] & 0xFFFFu) | ((uint32_t)x[3] << 16));
+                make_uint2(((uint32_t)x[0] & kLoMask) | (((uint32_t)x[1] & kLoMask) << 16),
+                           ((uint32_t)x[2] & kLoMask) | (((uint32_t)x[3] & kLoMask) << 16));
             *reinterpret_cast<uint32_t *>(sHi + e0) =
-                (((uint32_t)x[0] >> 16) & 0xFFu) | ((((uint32_t)x[1] >> 16) & 0xFFu) << 8) |
-                ((((uint32_t)x[2] >> 16) & 0xFFu) << 16) | ((((uint32_t)x[3] >> 16) & 0xFFu) << 24);
+                (((uint32_t)x[0] >> kLoBits) & 0xFFu) | ((((uint32_t)x[1] >> kLoBits) & 0xFFu) << 8) |
+                ((((uint32_t)x[2] >> kLoBits) & 0xFFu) << 16) | ((((uint32_t)x[3] >> kLoBits) & 0xFFu) << 24);
         }
         if (bad) atomicOr(a.status, kDevOverflow);
     }
@@ -199,7 +209,7 @@ loss_fast_kernel(const LossArgs a) {
             const long long n = a.counts[(int64_t)layer * E + i];
             const long long r = (long long)(E - 2 * K) * n + T * (long long)K;
             if (r > INT_MAX || r < 0) atomicOr(a.status, kDevOverflow);
-            if (kPlanes) s_r[i] = r;
+            if (kPlanes) s_rp[i] = (int)r;
             else sD[i * E + i] = -(int)r;
             if (a.n_zero && blockIdx.x == 0) a.n_zero[(int64_t)layer * E + i] = 0;
         }
@@ -227,10 +237,18 @@ loss_fast_kernel(const LossArgs a) {
     }
     __syncthreads();
 
-    double tok_sum = 0.0;
+    // sum of A_t over this lane's tokens as two fp32 (the fp64 unit is slow)
+    float tok_hi = 0.0f, tok_lo = 0.0f;
     for (; tb < t_end; tb += stride) {
         const int64_t t = tb + grp;
         const bool valid = t < t_end;
+        if constexpr (kPlanes) {  // two token groups ahead, on their way to L2
+            const int64_t tp = tb + 2 * stride;
+            if (lane < 16 && tp + (lane >> 3) < t_end)
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(zl + (tp + (lane >> 3)) * E + 32 * (lane & 7)));
+            else if (lane == 16 && tp < t_end)
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(il + tp * K));
+        }
         // prefetch the next token group
         const int64_t tn = tb + stride + grp;
         const int64_t tnc = (tn < t_end) ? tn : t_begin;
@@ -247,8 +265,9 @@ loss_fast_kernel(const LossArgs a) {
         for (int c = 0; c < 4; ++c) acc[c] = make_int4(0, 0, 0, 0);
         if constexpr (kPlanes) {
             uint32_t hp[4][2];  // high bytes of entries (0, 2) and (1, 3), 16-bit fields
+            uint32_t lp[4][2];  // low parts of entries (0, 1) and (2, 3), likewise (kNarrow)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) hp[c][0] = hp[c][1] = 0u;
+            for (int c = 0; c < 4; ++c) hp[c][0] = hp[c][1] = lp[c][0] = lp[c][1] = 0u;
 #pragma unroll
             for (int q = 0; q < K; ++q) {
                 const int base = js[q] * E + 4 * g;
@@ -256,36 +275,42 @@ loss_fast_kernel(const LossArgs a) {
                 for (int c = 0; c < 4; ++c) {
                     const uint2 lw = *reinterpret_cast<const uint2 *>(sLo + base + c * Q);
                     const uint32_t hw = *reinterpret_cast<const uint32_t *>(sHi + base + c * Q);
-                    acc[c].x += (int)(lw.x & 0xFFFFu);
-                    acc[c].y += (int)(lw.x >> 16);
-                    acc[c].z += (int)(lw.y & 0xFFFFu);
-                    acc[c].w += (int)(lw.y >> 16);
+                    if (kNarrow) {  // eight 13-bit values fit a 16-bit field
+                        lp[c][0] += lw.x;
+                        lp[c][1] += lw.y;
+                    } else {
+                        acc[c].x += (int)(lw.x & 0xFFFFu);
+                        acc[c].y += (int)(lw.x >> 16);
+                        acc[c].z += (int)(lw.y & 0xFFFFu);
+                        acc[c].w += (int)(lw.y >> 16);
+                    }
                     hp[c][0] += __byte_perm(hw, 0u, 0x4240);
                     hp[c][1] += __byte_perm(hw, 0u, 0x4341);
                 }
             }
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-                acc[c].x += (int)((hp[c][0] & 0xFFFFu) << 16);
-                acc[c].z += (int)(hp[c][0] & 0xFFFF0000u);
-                acc[c].y += (int)((hp[c][1] & 0xFFFFu) << 16);
-                acc[c].w += (int)(hp[c][1] & 0xFFFF0000u);
+                acc[c].x += (int)((lp[c][0] & 0xFFFFu) + ((hp[c][0] & 0xFFFFu) << kLoBits));
+                acc[c].y += (int)((lp[c][0] >> 16) + ((hp[c][1] & 0xFFFFu) << kLoBits));
+                acc[c].z += (int)((lp[c][1] & 0xFFFFu) + ((hp[c][0] >> 16) << kLoBits));
+                acc[c].w += (int)((lp[c][1] >> 16) + ((hp[c][1] >> 16) << kLoBits));
             }
-            // the diagonal of D': -R_j in the sum of each chosen expert j
+            // the diagonal of D': -R_j in the sum of each chosen expert j; bit
+            // 4 c + u: this lane's entry u of chunk c is chosen
+            uint32_t mine = 0u;
 #pragma unroll
             for (int q = 0; q < K; ++q) {
                 const int j = js[q];
-                if (((j & (Q - 1)) >> 2) != g) continue;
-                const int rj = (int)s_r[j];
-                const int cj = j / Q, ej = j & 3;
+                const uint32_t bit = 1u << (((j / Q) << 2) | (j & 3));
+                mine |= ((j & (Q - 1)) >> 2) == g ? bit : 0u;
+            }
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    if (c != cj) continue;
-                    acc[c].x -= ej == 0 ? rj : 0;
-                    acc[c].y -= ej == 1 ? rj : 0;
-                    acc[c].z -= ej == 2 ? rj : 0;
-                    acc[c].w -= ej == 3 ? rj : 0;
-                }
+            for (int c = 0; c < 4; ++c) {
+                const int4 r = *reinterpret_cast<const int4 *>(s_rp + c * Q + 4 * g);
+                acc[c].x -= (mine >> (4 * c)) & 1u ? r.x : 0;
+                acc[c].y -= (mine >> (4 * c + 1)) & 1u ? r.y : 0;
+                acc[c].z -= (mine >> (4 * c + 2)) & 1u ? r.z : 0;
+                acc[c].w -= (mine >> (4 * c + 3)) & 1u ? r.w : 0;
             }
         } else {
 #pragma unroll
@@ -342,7 +367,11 @@ loss_fast_kernel(const LossArgs a) {
         }
         const float inv = 1.0f / den;
         const float A = num * inv;
-        if (valid && g == 0) tok_sum += (double)A;
+        if (valid && g == 0) {  // Knuth's two-sum: the rounding error is kept in tok_lo
+            const float sum = __fadd_rn(tok_hi, A), b = __fsub_rn(sum, tok_hi);
+            tok_lo = __fadd_rn(tok_lo, __fadd_rn(__fsub_rn(tok_hi, __fsub_rn(sum, b)), __fsub_rn(A, b)));
+            tok_hi = sum;
+        }
         if (dzl && valid) {
             // dz = c/S * jac * (w - A) = jac * (cs w - cs A)
             const float cs = a.coef * inv;
@@ -366,6 +395,7 @@ loss_fast_kernel(const LossArgs a) {
         for (int q = 0; q < K; ++q) js[q] = jn[q];
     }
     // CTA partial, in warp and lane order
+    double tok_sum = (double)tok_hi + (double)tok_lo;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) tok_sum += __shfl_xor_sync(kFull, tok_sum, o);
     if (lane == 0) s_part[warp] = tok_sum;
@@ -395,7 +425,7 @@ loss_fast_kernel(const LossArgs a) {
             const int i = e / E, j = e - (e / E) * E;
             if (i != j) {
                 const long long d =
-                    kPlanes ? (long long)sLo[e] | ((long long)sHi[e] << 16) : (long long)sD[e];
+                    kPlanes ? (long long)sLo[e] | ((long long)sHi[e] << kLoBits) : (long long)sD[e];
                 o += d * d;
             }
         }
@@ -466,11 +496,10 @@ idx_from_bits_kernel(const uint32_t *__restrict__ bits, int64_t T, int64_t W, in
     }
 }
 
-template <int E, int K, bool kRFromCounts>
-cudaError_t run_loss_fast(const LossArgs &args, int gate, int P, const Problem &p, cudaStream_t s) {
+template <int E, int K, int kGate, bool kRFromCounts, bool kNarrow>
+cudaError_t run_loss_fast(const LossArgs &args, int P, const Problem &p, cudaStream_t s) {
     const size_t smem = loss_fast_smem<E>();
-    cudaError_t e = ensure_smem_limit<loss_fast_kernel<E, K, 0, kRFromCounts>>(smem);
-    if (e == cudaSuccess) e = ensure_smem_limit<loss_fast_kernel<E, K, 1, kRFromCounts>>(smem);
+    cudaError_t e = ensure_smem_limit<loss_fast_kernel<E, K, kGate, kRFromCounts, kNarrow>>(smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)P, (unsigned)p.L);
@@ -482,17 +511,27 @@ cudaError_t run_loss_fast(const LossArgs &args, int gate, int P, const Problem &
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (gate == 0) return cudaLaunchKernelEx(&cfg, loss_fast_kernel<E, K, 0, kRFromCounts>, args);
-    return cudaLaunchKernelEx(&cfg, loss_fast_kernel<E, K, 1, kRFromCounts>, args);
+    return cudaLaunchKernelEx(&cfg, loss_fast_kernel<E, K, kGate, kRFromCounts, kNarrow>, args);
+}
+
+template <int E, int K, bool kRFromCounts>
+cudaError_t dispatch_loss_gate(const LossArgs &args, int gate, int P, const Problem &p, cudaStream_t s) {
+    if constexpr (E == 256) {
+        if (p.T < (1 << 21))
+            return gate == 0 ? run_loss_fast<E, K, 0, kRFromCounts, true>(args, P, p, s)
+                             : run_loss_fast<E, K, 1, kRFromCounts, true>(args, P, p, s);
+    }
+    return gate == 0 ? run_loss_fast<E, K, 0, kRFromCounts, false>(args, P, p, s)
+                     : run_loss_fast<E, K, 1, kRFromCounts, false>(args, P, p, s);
 }
 
 template <int E, bool kRFromCounts>
 cudaError_t dispatch_loss_k(const LossArgs &args, int gate, int P, const Problem &p, cudaStream_t s) {
     switch (p.k) {
-        case 1: return run_loss_fast<E, 1, kRFromCounts>(args, gate, P, p, s);
-        case 2: return run_loss_fast<E, 2, kRFromCounts>(args, gate, P, p, s);
-        case 4: return run_loss_fast<E, 4, kRFromCounts>(args, gate, P, p, s);
-        default: return run_loss_fast<E, 8, kRFromCounts>(args, gate, P, p, s);
+        case 1: return dispatch_loss_gate<E, 1, kRFromCounts>(args, gate, P, p, s);
+        case 2: return dispatch_loss_gate<E, 2, kRFromCounts>(args, gate, P, p, s);
+        case 4: return dispatch_loss_gate<E, 4, kRFromCounts>(args, gate, P, p, s);
+        default: return dispatch_loss_gate<E, 8, kRFromCounts>(args, gate, P, p, s);
     }
 }
 

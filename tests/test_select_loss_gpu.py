@@ -155,6 +155,25 @@ def test_routing_gradient(dl, T, k):
                extra=oracle.route_backward(zl, ids, gl), extra_bound=route_bound(zl, ids, gl, 0))
 
 
+# E = 256: 13-bit and (from T = 2^21 on) 16-bit fields of D in shared memory,
+# against the general kernels, which take logits that are not 16-byte aligned.
+# Both sides are within the bound above; an entry of dz is at most p_max (|w| + M).
+@pytest.mark.parametrize("T,k,gate", [(1, 8, 0), (4097, 8, 1), (70001, 4, 0), (1 << 21, 8, 0)])
+def test_planes_against_general_path(dl, T, k, gate):
+    E = 256
+    z = workloads.random_logits(T, E, seed=T, device="cuda")
+    z[:, :, :4] += 6.0                               # crowded experts: large counts
+    shifted = torch.empty(T * E + 1, device="cuda")[1:].view(1, T, E)
+    shifted.copy_(z)
+    a, b = dl.forward_backward(z, k, gate), dl.forward_backward(shifted, k, gate)
+    torch.cuda.synchronize()
+    assert dl.device_status(a.workspace) == 0 and dl.device_status(b.workspace) == 0
+    assert torch.equal(a.bits, b.bits) and torch.equal(a.D, b.D) and torch.equal(a.counts, b.counts)
+    tol = 4.0 * (E + 64) * U
+    assert float(a.loss) == pytest.approx(float(b.loss), rel=tol, abs=tol)
+    assert (a.dlogits - b.dlogits).abs().max() <= 2 * tol * b.dlogits.abs().max()
+
+
 # the narrow workspace layout: E = 256 in the library's fixed 16 MiB array where
 # the layout with counts does not fit any more
 @pytest.mark.parametrize("T", [1 << 16, 500000])
