@@ -115,17 +115,16 @@ def measured_peaks():
 # The sources each timed unit's kernels are compiled from (its launcher and
 # argument checks included); a traffic record holds only while they are
 # unchanged.
+SELECT_SOURCES = ["sig_fast.cuh", "sig_fast.cu", "select.cuh", "select.cu", "topk_net.cuh"]
+LOSS_SOURCES = ["loss_mma.cuh", "loss_mma.cu", "loss_mma_nb1.cu", "loss_mma_nb2.cu", "loss_mma_nb3.cu",
+                "loss_mma_nb4.cu", "loss_fast.cu", "loss.cu"]
+HOST_SOURCES = ["tma.cuh", "tma_host.cu", "dol_internal.cuh", "api.cu"]
 UNIT_SOURCES = {
-    "do_forward_backward": ["sig_fast.cuh", "sig_fast.cu", "cooc_reduce.cu", "loss_mma.cu",
-                            "loss.cu", "tma.cuh", "tma_host.cu", "dol_internal.cuh", "api.cu"],
-    "do_routing": ["sig_fast.cuh", "route.cu", "signatures.cu", "tma.cuh", "tma_host.cu",
-                   "dol_internal.cuh", "api.cu"],
+    "do_forward_backward": SELECT_SOURCES + ["cooc_reduce.cu"] + LOSS_SOURCES + HOST_SOURCES,
+    "do_routing": SELECT_SOURCES + ["route.cu", "signatures.cu"] + HOST_SOURCES,
     "do_route_backward": ["route_bwd.cu", "dol_internal.cuh", "api.cu"],
-    "do_routed_backward": ["loss_mma.cu", "route_bwd.cu", "tma.cuh", "tma_host.cu",
-                           "dol_internal.cuh", "api.cu"],
-    "do_router_forward_backward": ["router.cu", "sig_fast.cuh", "cooc_reduce.cu", "loss_mma.cu",
-                                   "loss.cu", "tma.cuh", "tma_host.cu", "dol_internal.cuh",
-                                   "api.cu"],
+    "do_routed_backward": LOSS_SOURCES + ["route_bwd.cu"] + HOST_SOURCES,
+    "do_router_forward_backward": ["router.cu", "topk_net.cuh", "cooc_reduce.cu"] + LOSS_SOURCES + HOST_SOURCES,
 }
 
 

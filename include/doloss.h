@@ -144,12 +144,13 @@ do_status do_loss_fwd_bwd(const float *logits, const uint32_t *bits, const int32
 
 /* Steps 1-3 in one call on a local window (d_scale = 1): logits in; bits,
  * counts, D, loss, origin_do (may be NULL) and dlogits (may be NULL) out.
- * With E = 128, the sigmoid-normalised gate, k in {1, 2, 4, 8}, T <= 66052
- * and dlogits given, the gradient pass computes V = F D' on the tensor cores
- * (F the one-hot selections, D' = D with -R on the diagonal); elsewhere it
- * gathers rows of D' on the ALU (as do_loss_fwd_bwd always does; at E = 256,
- * k in {1, 2, 4, 8}, T < 2^24 and 16-byte aligned logits, D and dlogits with
- * D held in 24-bit shared-memory planes).  The two agree within the stated
+ * With E <= 128 a multiple of 4, k <= 16, T < 2^22 and 16-byte aligned logits
+ * and dlogits, the gradient pass (here and in do_loss_fwd_bwd) computes V = F D'
+ * on the tensor cores (F the one-hot selections, D' = D with -R on the
+ * diagonal); elsewhere, and where few choices or tokens make that the faster
+ * way, it gathers rows of D' on the ALU (at E = 256, k in {1, 2, 4, 8},
+ * T < 2^24 and 16-byte aligned logits, D and dlogits with D held in
+ * shared-memory planes of 21 or 24 bits).  The two agree within the stated
  * tolerances. */
 do_status do_forward_backward(const float *logits, int64_t T, int32_t E, int32_t k, int32_t L,
                               int32_t gate, float grad_scale, uint32_t *bits, int32_t *counts,
@@ -177,8 +178,9 @@ do_status do_forward_backward(const float *logits, int64_t T, int32_t E, int32_t
  * NULL.  All are exact integers except combine, which is fp32 (a few ulp of
  * the exact ratio); all are identical run to run.  Needs T k <= INT32_MAX
  * (DO_ERR_UNSUPPORTED otherwise).  16-byte aligned logits, expert_ids and
- * combine with E in {32, 64, 128} and k in {1, 2, 4, 8} take the fast
- * selection kernel.  workspace: do_routing_workspace_size(T, E, k, L) bytes
+ * combine with E in {32, 64, 128} and k in {1, 2, 4, 8}, and 16-byte aligned
+ * logits with any E <= 512 that is a multiple of 4 and k <= 16, take the fast
+ * selection kernels.  workspace: do_routing_workspace_size(T, E, k, L) bytes
  * of device memory, 256-byte aligned, zero-filled before its first use (it
  * holds the device status word, read by do_device_status, and the
  * signatures).  Asynchronous on `stream`. */
@@ -211,16 +213,15 @@ size_t do_routing_workspace_size(int64_t T, int32_t E, int32_t k, int32_t L);
  * it wrote.  With d_scale = 1, D is the forward half's matrix; otherwise D
  * is a matrix summed over data-parallel ranks or micro-batches that include
  * these tokens (Eq. global_do, d_scale = 1 / their number) and m stays T.
- * With E = 128, the sigmoid-normalised gate, k in {1, 2, 4, 8} and 16-byte
- * aligned logits, D, bits, dlogits, expert_ids and grad_combine, the
- * tensor-core loss kernel runs and adds the routing gradient in its
- * epilogue: with d_scale = 1 (and T <= 66052) from the image of D' the
- * forward half left; otherwise a kernel first builds the image of the given
- * matrix and checks, per problem, that its two fp16 pieces hold it exactly
- * (0 <= D_ij < 2^22 off the diagonal, D_ii = 0, row sums below 2^23), and
- * the problems that fail the check go to the ALU loss kernel and the
- * routing-gradient kernel instead.  Elsewhere the ALU loss kernels run and a
- * second kernel adds the routing gradient.  The result agrees with
+ * The loss kernels are do_forward_backward's.  With the tensor-core one and
+ * d_scale = 1 the image of D' is the one the forward half left; otherwise a
+ * kernel first builds the image of the given matrix and checks, per problem,
+ * that its two fp16 pieces hold it exactly (0 <= D_ij < 2^22 off the diagonal,
+ * D_ii = 0, row sums within int32); the problems that fail the check have
+ * their rows gathered from D.  With E = 128, the sigmoid-normalised gate,
+ * k in {1, 2, 4, 8} and 16-byte aligned expert_ids and grad_combine the
+ * tensor-core kernel adds the routing gradient in its epilogue, elsewhere a
+ * second kernel does.  The result agrees with
  * do_loss_fwd_bwd's dlogits plus do_route_backward's within the sum of their
  * tolerances.
  *
@@ -377,9 +378,11 @@ do_status do_forward_backward_host_async(const float *h_logits, int64_t T, int32
  * interface variant of steps 1-3, with the same arguments and results as
  * do_forward_backward except that the workspace is a fixed 16 MiB array
  * inside the library, one per device.
- *  - Sizes whose do_workspace_size exceeds DO_STATIC_SCRATCH_BYTES are
- *    rejected with DO_ERR_WORKSPACE before anything is launched (for
- *    E = 128, k = 8, L = 1 that is T above about 0.97 million tokens).
+ *  - Sizes whose workspace exceeds DO_STATIC_SCRATCH_BYTES are rejected with
+ *    DO_ERR_WORKSPACE before anything is launched (for E = 128, k = 8, L = 1
+ *    that is T above about 0.97 million tokens).  Where do_workspace_size asks
+ *    for more than that only for the co-occurrence counts and the operand image
+ *    (E not in {32, 64, 128}), the call runs without them.
  *  - Unlike the other entry points it keeps state: the first call in a CUDA
  *    context (with its device current) looks up the array's device address
  *    and caches it for that context (a context created later, e.g. after

@@ -181,7 +181,10 @@ do_status do_loss_fwd_bwd(const float *logits, const uint32_t *bits, const int32
     uint8_t *idx = reinterpret_cast<uint8_t *>(ws + w.idx);
     long long *origin = reinterpret_cast<long long *>(origin_do);
     cudaError_t e = cudaSuccess;
-    if (w.image && dol::loss_mma_supported(p, logits, dlogits) && aligned(D, 16)) {
+    const bool alu = dol::loss_fast_supported(p, logits, D, dlogits) && aligned(bits, 16);
+    // (the fused call's kernel: the same results bit for bit)
+    if (w.image && dol::loss_mma_supported(p, logits, dlogits) && aligned(D, 16) &&
+        !(alu && dol::loss_alu_faster(p, gate))) {
         // the given matrix's image of D' and origin_do, then the tensor-core kernel
         unsigned char *bimg = reinterpret_cast<unsigned char *>(ws + w.bimg);
         int *img_ok = reinterpret_cast<int *>(ws + w.img_ok);
@@ -192,7 +195,7 @@ do_status do_loss_fwd_bwd(const float *logits, const uint32_t *bits, const int32
                                      img_ok, D);
         return from_cuda(e);
     }
-    if (dol::loss_fast_supported(p, logits, D, dlogits) && aligned(bits, 16)) {
+    if (alu) {
         e = dol::launch_idx_from_bits(bits, p, idx, done, p.L, s);
         if (e == cudaSuccess)
             e = dol::launch_loss_fast(logits, idx, D, nullptr, nullptr, p, gate, d_scale, grad_scale,
@@ -244,7 +247,8 @@ do_status forward_backward_impl(const float *logits, int64_t T, int32_t E, int32
     const bool loss_idx = select && aligned(bits, 16) &&
                           (dol::loss_fast_supported(p, logits, D, dlogits) ||
                            dol::loss_fast256_supported(p, logits, D, dlogits));
-    const bool mma = select && w.image && dol::loss_mma_supported(p, logits, dlogits);
+    const bool mma = select && w.image && dol::loss_mma_supported(p, logits, dlogits) &&
+                     !(loss_idx && dol::loss_alu_faster(p, gate));
     // (the tensor-core one where it is cheap for the selection to write them)
     const bool use_idx = loss_idx && (!mma || dol::signatures_fast_supported(logits, p));
     uint8_t *idx = use_idx ? reinterpret_cast<uint8_t *>(ws + w.idx) : nullptr;
@@ -462,7 +466,10 @@ do_status do_routed_backward(const float *logits, int64_t T, int32_t E, int32_t 
     // forward half left for the tensor-core kernel; otherwise D is a matrix
     // summed over ranks or micro-batches (Eq. global_do), read as given.
     const bool local = d_scale == 1.0f;
-    const bool mma = split_mma(p, logits, w) && dol::loss_mma_supported(p, logits, dlogits);
+    const bool have_idx = dol::signatures_fast_supported(logits, p);
+    const bool alu = split_fast(p, logits, bits, D) && aligned(dlogits, 16);
+    const bool mma = split_mma(p, logits, w) && dol::loss_mma_supported(p, logits, dlogits) &&
+                     !(alu && dol::loss_alu_faster(p, gate));
     unsigned char *bimg = reinterpret_cast<unsigned char *>(ws + w.bimg);
     cudaError_t e;
     if (mma && (local || aligned(D, 16))) {
@@ -471,7 +478,6 @@ do_status do_routed_backward(const float *logits, int64_t T, int32_t E, int32_t 
         e = local ? cudaSuccess : dol::launch_dprime_image(D, p, bimg, img_ok, nullptr, nullptr, s);
         // the routing gradient is added in the loss kernel's epilogue where it
         // can, else by its own kernel
-        const bool have_idx = dol::signatures_fast_supported(logits, p);
         const bool rg_mma = rg && have_idx && dol::loss_mma_route_grad(p, gate, expert_ids, grad_combine);
         if (e == cudaSuccess)
             e = dol::launch_loss_mma(logits, bits, have_idx ? idx : nullptr, bimg, local ? n_acc : nullptr, p, gate, d_scale,
@@ -479,7 +485,7 @@ do_status do_routed_backward(const float *logits, int64_t T, int32_t E, int32_t 
                                      rg_mma ? expert_ids : nullptr, rg_mma ? grad_combine : nullptr,
                                      img_ok, local ? nullptr : D);
         if (rg_mma) return from_cuda(e);
-    } else if (split_fast(p, logits, bits, D) && aligned(dlogits, 16)) {
+    } else if (alu) {
         e = dol::launch_idx_from_bits(bits, p, idx, nullptr, 0, s);
         // the row sums of D come from the counts only for the local matrix
         if (e == cudaSuccess)

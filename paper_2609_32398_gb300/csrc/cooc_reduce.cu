@@ -19,10 +19,11 @@
 namespace dol {
 namespace {
 
-// 256 threads, 32 registers: two CTAs fit on an SM beside a selection CTA
-// (46 K registers, 221 KB), so the reduction is resident and set up when the
-// selection ends; CTAs of 1024 threads started only after it (36.4 against
-// 3X.X us for the E = 128, T = 65536 step).
+// Bound by L2 latency (1.75 us of the E = 128, T = 65536 step, whose partials are
+// 5 MB).  256 threads with 20 loads in flight: with 128, 512 and 1024 threads the
+// step took 30.5, 31.0 and 31.1 against 30.2 us (the routed step with 1024: 55.8
+// against 52.4), and with the search for (a, b) moved ahead of the dependency wait
+// 31.3.
 constexpr int kRedWarps = 8;
 constexpr int kRedThreads = kRedWarps * 32;
 constexpr int kRedLoads = 20;  // partials a warp requests at once

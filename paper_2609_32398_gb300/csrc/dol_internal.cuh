@@ -197,6 +197,7 @@ cudaError_t launch_idx_from_bits(const uint32_t *bits, const Problem &p, uint8_t
 // null (forward only).
 bool loss_mma_supported(const Problem &p, const float *logits, const float *dlogits);
 bool loss_mma_big(const Problem &p);
+bool loss_alu_faster(const Problem &p, int gate);
 bool loss_mma_route_grad(const Problem &p, int gate, const int *ids, const float *g);
 // idx (may be null; k in {1, 2, 4, 8}, E in {32, 64, 128}; needed for the routing
 // gradient): the chosen experts of every token, as the selection wrote them.

@@ -29,6 +29,24 @@ bool loss_mma_supported(const Problem &p, const float *logits, const float *dlog
 // R_i <= (E - 1) T may reach 2^23: the marker diagonal.
 bool loss_mma_big(const Problem &p) { return (int64_t)(p.E - 1) * p.T >= (int64_t)(1 << 23); }
 
+// Where the ALU kernel of loss_fast.cu (E in {32, 64, 128}, k in {1, 2, 4, 8}) is
+// the faster one: its gather of k rows a token costs by k T, the tensor-core
+// kernel's set-up (TMEM, the operand image, a first MMA) once.  Measured, step
+// with the ALU kernel against the tensor cores, us:
+//   k T <= 512 E   E = 64,  k = 8, T = 4096:  10.8 / 11.4   (T = 8192: 11.9 / 11.5)
+//                  E = 128, k = 8, T = 8192:  15.0 / 15.1   (T = 16384: 18.3 / 16.7)
+//                  E = 32,  k = 2, T = 8192:   8.9 /  9.1   (T = 16384: 9.9 / 9.8)
+//   k <= E / 64    E = 64,  k = 1, T = 200000: 30.9 / 32.6
+//                  E = 128, k = 2, T = 93176:  30.6 / 33.9  (T = 200000: 61.3 / 60.3)
+// At E = 128, sigmoid-norm, the tensor cores add the routing gradient as well, so
+// the smaller sizes stay with them.
+bool loss_alu_faster(const Problem &p, int gate) {
+    const bool sizes = (p.E == 32 || p.E == 64 || p.E == 128) && (p.k == 1 || p.k == 2 || p.k == 4 || p.k == 8);
+    if (!sizes || (p.E == 128 && gate == 0 && !loss_mma_big(p))) return false;
+    const int64_t tokens = p.T * p.L;
+    return tokens * p.k <= 512 * (int64_t)p.E || (p.k <= p.E / 64 && (p.E == 64 || tokens <= (1 << 17)));
+}
+
 // The routing gradient is added in the epilogue (else by its own kernel).
 bool loss_mma_route_grad(const Problem &p, int gate, const int *ids, const float *g) {
     auto al = [](const void *q) { return reinterpret_cast<uintptr_t>(q) % 16 == 0; };

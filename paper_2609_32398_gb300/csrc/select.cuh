@@ -40,12 +40,11 @@
 namespace dol {
 
 constexpr int kSelMaxSlots = 16;
-// Most teams (pairs of consumer warps) and block size for lists of KP values:
-// the launch bound keeps 72 registers a thread for KP <= 8, so that the
-// reduction's CTAs fit beside 640 threads.
+// Most teams (pairs of consumer warps) and block size for lists of KP values
+// (the launch bound of 896 threads keeps 72 registers a thread for KP <= 8).
 constexpr int sel_max_teams(int KP) { return KP <= 8 ? 9 : 6; }
 constexpr int sel_threads(int KP) { return (2 * sel_max_teams(KP) + 2) * 32; }
-// Leaves room for two CTAs of the reduction kernel on the SM.
+// Leaves room for two small CTAs of the next kernel on the SM.
 constexpr int kSelMaxSmem = 226304;
 
 // Shared memory of one launch: ring | barriers and flags | lists | masks | counters.
