@@ -1,7 +1,6 @@
-// Step 3 for k in {1, 2, 4, 8} where the tensor-core kernel (loss_mma.cuh) does
-// not apply: E = 256, and E in {32, 64, 128} from T = 2^22 on or without room for
-// its image of D'.  The
-// surrogate DO-loss and its gradient (Sec. 3.1.3, Eq. do_loss; Eq. global_do
+// Step 3 on the ALU for k in {1, 2, 4, 8}: E = 256, and E in {32, 64, 128} where
+// the tensor-core kernel is the slower one (loss_alu_faster) or does not apply
+// (T >= 2^22, no room for its image of D').  The surrogate DO-loss and its gradient (Sec. 3.1.3, Eq. do_loss; Eq. global_do
 // scaling).
 //
 // With R_i = sum_j D_ij, put D'_ij = D_ij off the diagonal and D'_ii = -R_i.

@@ -12,7 +12,8 @@ one ex2.approx (2 ulp) of a product rounded at |z| <= 8 (12 u) and one rcp.appro
 (1 ulp), so s, the sums and their quotient are within (E + 64) u; the integers
 behind w are exact below 2^24 and rounded once above.  So
   |dz - ref| <= 2 (E + 64) u p (1 - s) (|w| + M_t),  |loss - ref| <= 2 (E + 64) u sum_t M_t,
-the factor 2 for the two factors of the product.  u p_max max|w| is added for
+the factor 2 for the two factors of the product (at E <= 64 and in the gather kernel
+1 - s comes as s - s^2, within u / (1 - s) <= 150 u at z <= 5, inside the same bound).  u p_max max|w| is added for
 results rounded near zero.
 """
 import numpy as np
@@ -85,6 +86,8 @@ def test_selection(dl, T, E, k, L, ties):
         assert np.array_equal(r.pos[l].cpu().numpy(), pos)
 
 
+# both sides of the line between the gather and the tensor-core kernel (k T L =
+# 512 E; E = 128: two choices at the marker's sizes);
 # one to four boxes of the tensor-core kernel, padded and whole; tiles of 128
 # tokens and their remainders; both gates; the marker diagonal ((E - 1) T >=
 # 2^23); counted widths above 128 and the generic kernel (k > 64, E > 256)
@@ -92,6 +95,8 @@ def test_selection(dl, T, E, k, L, ties):
     (1, 4, 1, 1, 0), (127, 12, 3, 2, 1), (129, 32, 16, 1, 0), (1300, 36, 4, 1, 1), (128, 64, 5, 3, 0),
     (641, 68, 7, 1, 0), (255, 96, 6, 2, 1), (20011, 100, 8, 1, 0), (385, 128, 10, 2, 1),
     (2000, 128, 3, 1, 0), (66053, 128, 5, 1, 0), (84737, 100, 8, 1, 1),
+    (4096, 64, 8, 1, 0), (4097, 64, 8, 1, 1), (16384, 32, 1, 1, 1), (16385, 32, 1, 1, 0),
+    (2049, 128, 4, 2, 1), (66053, 128, 2, 1, 0),
     (300, 132, 8, 1, 0), (777, 160, 16, 2, 1), (1000, 252, 3, 1, 0),
     (130, 100, 70, 2, 1), (99, 300, 5, 1, 0), (4099, 320, 9, 2, 1), (33, 1000, 12, 1, 0)])
 def test_step(dl, T, E, k, L, gate):
