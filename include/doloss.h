@@ -131,7 +131,9 @@ do_status do_accumulate_distances(const int32_t *D, int32_t E, int32_t L, int32_
  * (Eq. origin_do; may be NULL) and dlogits [L][T][E] = grad_scale * dL/dz
  * (may be NULL for a forward-only call).  bits must hold the selection that
  * produced the token rows of logits; D may come from any source whose row
- * sums fit int32.  workspace: do_workspace_size(T, E, k, L) bytes of device
+ * sums fit int32.  Logits are finite; with the sigmoid-normalised gate a
+ * token's weights p = s / sum(s) are relative to its own sum, exact to fp32
+ * rounding while its largest logit is above -80.  workspace: do_workspace_size(T, E, k, L) bytes of device
  * memory, 256-byte aligned and zero-filled before its first use (cudaMemset);
  * every call leaves it ready for the next one.  A workspace serves one call
  * at a time; after a call fails or do_device_status reports an error, zero it
