@@ -190,7 +190,7 @@ do_status do_loss_fwd_bwd(const float *logits, const uint32_t *bits, const int32
         int *img_ok = reinterpret_cast<int *>(ws + w.img_ok);
         e = dol::launch_dprime_image(D, p, bimg, img_ok, origin, done, s);
         if (e == cudaSuccess)
-            e = dol::launch_loss_mma(logits, bits, nullptr, bimg, nullptr, p, gate, d_scale, grad_scale, loss,
+            e = dol::launch_loss_mma(logits, bits, nullptr, bimg, p, gate, d_scale, grad_scale, loss,
                                      dlogits, partials, done, status, nullptr, s, nullptr, nullptr,
                                      img_ok, D);
         return from_cuda(e);
@@ -198,7 +198,7 @@ do_status do_loss_fwd_bwd(const float *logits, const uint32_t *bits, const int32
     if (alu) {
         e = dol::launch_idx_from_bits(bits, p, idx, done, p.L, s);
         if (e == cudaSuccess)
-            e = dol::launch_loss_fast(logits, idx, D, nullptr, nullptr, p, gate, d_scale, grad_scale,
+            e = dol::launch_loss_fast(logits, idx, D, nullptr, p, gate, d_scale, grad_scale,
                                       loss, origin, dlogits, partials, done, status, nullptr, s);
         return from_cuda(e);
     }
@@ -257,12 +257,10 @@ do_status forward_backward_impl(const float *logits, int64_t T, int32_t E, int32
                  dol::router_supported(p, rin->H, rin->X, rin->Wr, logits)))
         return DO_ERR_UNSUPPORTED;
     cudaError_t e;
-    int *n_acc = nullptr;
     if (select && w.cooc) {
         // signatures + per-CTA co-occurrence counts -> reduction, which builds
         // D = n_i + n_j - 2 c_ij and writes D, the counts and origin_do
         uint32_t *parts = reinterpret_cast<uint32_t *>(ws + w.cooc_parts);
-        n_acc = reinterpret_cast<int *>(ws + w.n_acc);
         // origin_do is summed by the reduction kernel (integer atomics) and
         // status_out ORed by the loss kernel: zero them first
         const dol::ZeroSpans zero = {{done, reinterpret_cast<int *>(origin_do), status_out},
@@ -270,15 +268,15 @@ do_status forward_backward_impl(const float *logits, int64_t T, int32_t E, int32
                                       status_out ? 1 : 0}};
         const bool big = dol::loss_mma_big(p);
         unsigned char *bimg = mma ? reinterpret_cast<unsigned char *>(ws + w.bimg) : nullptr;
-        const dol::SelectOut so = {bits, n_acc, idx, parts, zero, status, route};
+        const dol::SelectOut so = {bits, nullptr, idx, parts, zero, status, route};
         e = rin ? dol::launch_router_signatures(rin->X, rin->Wr, rin->H, const_cast<float *>(logits),
-                                                p, bits, n_acc, idx, parts, zero, status, s)
+                                                p, bits, idx, parts, zero, status, s)
                 : dol::launch_select(logits, p, so, s);
         const int P1 = rin ? dol::router_ctas_per_problem(p) : dol::sig_ctas_per_problem(p);
         if (e == cudaSuccess)
-            e = dol::launch_cooc_reduce(parts, P1, n_acc, p, D, counts, bimg, big, origin, s);
+            e = dol::launch_cooc_reduce(parts, P1, p, D, counts, bimg, big, origin, s);
         if (e == cudaSuccess && mma) {
-            e = dol::launch_loss_mma(logits, bits, idx, bimg, n_acc, p, gate, 1.0f, grad_scale, loss, dlogits,
+            e = dol::launch_loss_mma(logits, bits, idx, bimg, p, gate, 1.0f, grad_scale, loss, dlogits,
                                      partials, done, status, status_out, s);
             if (e == cudaSuccess && status_done) *status_done = status_out != nullptr;
             if (e == cudaSuccess && ra)
@@ -301,12 +299,12 @@ do_status forward_backward_impl(const float *logits, int64_t T, int32_t E, int32
     }
     if (e == cudaSuccess) {
         if (loss_idx) {
-            e = dol::launch_loss_fast(logits, idx, D, counts, n_acc, p, gate, 1.0f, grad_scale,
+            e = dol::launch_loss_fast(logits, idx, D, counts, p, gate, 1.0f, grad_scale,
                                       loss, origin, dlogits, partials, done, status, status_out, s);
             if (e == cudaSuccess && status_done) *status_done = status_out != nullptr;
         } else {
             e = dol::launch_loss(logits, bits, D, p, gate, 1.0f, grad_scale, loss, origin, dlogits,
-                                 status, partials, s, counts, n_acc);
+                                 status, partials, s, counts);
         }
     }
     // the dispatch order (from the signatures and ids alone) follows the loss kernel
@@ -401,11 +399,9 @@ do_status do_routed_forward(const float *logits, int64_t T, int32_t E, int32_t k
     int *rscratch = reinterpret_cast<int *>(ws + w.route_base);
     const dol::RouteOut route = {expert_ids, combine, gate};
     cudaError_t e = cudaSuccess;
-    int *n_acc = nullptr;
     if (dol::select_supported(logits, p) && w.cooc) {
         int *done = reinterpret_cast<int *>(ws + w.done);
         uint32_t *parts = reinterpret_cast<uint32_t *>(ws + w.cooc_parts);
-        n_acc = reinterpret_cast<int *>(ws + w.n_acc);
         const dol::ZeroSpans zero = {{done, reinterpret_cast<int *>(origin_do), nullptr},
                                      {(int64_t)p.L, origin_do ? 2 * (int64_t)p.L : 0, 0}};
         // what the backward half's loss kernel reads
@@ -413,10 +409,10 @@ do_status do_routed_forward(const float *logits, int64_t T, int32_t E, int32_t k
                                   ? reinterpret_cast<unsigned char *>(ws + w.bimg) : nullptr;
         uint8_t *idx = dol::signatures_fast_supported(logits, p)
                            ? reinterpret_cast<uint8_t *>(ws + w.idx) : nullptr;
-        const dol::SelectOut so = {bits, n_acc, idx, parts, zero, reinterpret_cast<int *>(ws), route};
+        const dol::SelectOut so = {bits, nullptr, idx, parts, zero, reinterpret_cast<int *>(ws), route};
         e = dol::launch_select(logits, p, so, s);
         if (e == cudaSuccess)
-            e = dol::launch_cooc_reduce(parts, dol::sig_ctas_per_problem(p), n_acc, p, D,
+            e = dol::launch_cooc_reduce(parts, dol::sig_ctas_per_problem(p), p, D,
                                         counts, bimg, dol::loss_mma_big(p),
                                         reinterpret_cast<long long *>(origin_do), s);
     } else {
@@ -425,11 +421,9 @@ do_status do_routed_forward(const float *logits, int64_t T, int32_t E, int32_t k
         if (e == cudaSuccess && origin_do)
             e = dol::launch_origin_do(D, p, reinterpret_cast<long long *>(origin_do), s);
     }
-    // no loss kernel follows in this call: the dispatch kernels clear the
-    // counts accumulator
     if (e == cudaSuccess)
         e = dol::launch_route_dispatch(bits, expert_ids, p, expert_offsets, dispatch_rows,
-                                       dispatch_pos, rscratch, s, n_acc);
+                                       dispatch_pos, rscratch, s);
     return from_cuda(e);
 }
 
@@ -460,7 +454,6 @@ do_status do_routed_backward(const float *logits, int64_t T, int32_t E, int32_t 
     int *status = reinterpret_cast<int *>(ws);
     int *done = reinterpret_cast<int *>(ws + w.done);
     uint8_t *idx = reinterpret_cast<uint8_t *>(ws + w.idx);
-    int *n_acc = reinterpret_cast<int *>(ws + w.n_acc);
     double *partials = reinterpret_cast<double *>(ws + w.partials);
     // d_scale = 1: D is the forward half's own matrix, whose fp16 image the
     // forward half left for the tensor-core kernel; otherwise D is a matrix
@@ -480,7 +473,7 @@ do_status do_routed_backward(const float *logits, int64_t T, int32_t E, int32_t 
         // can, else by its own kernel
         const bool rg_mma = rg && have_idx && dol::loss_mma_route_grad(p, gate, expert_ids, grad_combine);
         if (e == cudaSuccess)
-            e = dol::launch_loss_mma(logits, bits, have_idx ? idx : nullptr, bimg, local ? n_acc : nullptr, p, gate, d_scale,
+            e = dol::launch_loss_mma(logits, bits, have_idx ? idx : nullptr, bimg, p, gate, d_scale,
                                      grad_scale, loss, dlogits, partials, done, status, nullptr, s,
                                      rg_mma ? expert_ids : nullptr, rg_mma ? grad_combine : nullptr,
                                      img_ok, local ? nullptr : D);
@@ -489,7 +482,7 @@ do_status do_routed_backward(const float *logits, int64_t T, int32_t E, int32_t 
         e = dol::launch_idx_from_bits(bits, p, idx, nullptr, 0, s);
         // the row sums of D come from the counts only for the local matrix
         if (e == cudaSuccess)
-            e = dol::launch_loss_fast(logits, idx, D, local ? counts : nullptr, n_acc, p, gate,
+            e = dol::launch_loss_fast(logits, idx, D, local ? counts : nullptr, p, gate,
                                       d_scale, grad_scale, loss, nullptr, dlogits, partials, done,
                                       status, nullptr, s);
     } else {
@@ -532,7 +525,7 @@ do_status do_routing(const float *logits, int64_t T, int32_t E, int32_t k, int32
         e = dol::launch_select(logits, p, so, s);
         if (e == cudaSuccess)
             e = dol::launch_route_dispatch(bits, expert_ids, p, expert_offsets, dispatch_rows,
-                                           dispatch_pos, rscratch, s, nullptr, counts);
+                                           dispatch_pos, rscratch, s, counts);
         return from_cuda(e);
     }
     e = dol::launch_signatures(logits, p, bits, counts, s, route);

@@ -1,10 +1,10 @@
-// Reduction of the per-CTA co-occurrence triangles of the fused path.
-//   c_ab = sum_t f_at f_bt, c_aa = n_a, and the Hamming distance
-//   D_ab = n_a + n_b - 2 c_ab                                   (App. C.3)
-// and, alongside, Eq. origin_do: sum over a != b of D_ab^2 (exact integer
+// Reduction of the selection CTAs' triangles of distances (tri_chunk): the
+// Hamming distance
+//   D_ab = n_a + n_b - 2 c_ab, c_ab = sum_t f_at f_bt           (App. C.3)
+// is a sum over tokens, and so the sum of the CTAs' own; the diagonal holds 2 n_a.
+// Alongside, Eq. origin_do: sum over a != b of D_ab^2 (exact integer
 // adds, one per CTA).
-// The counts n_a were already summed (one atomic per expert and CTA) by the
-// signatures kernel.  A CTA owns 32 consecutive triangle words; its warps
+// A CTA owns 32 consecutive triangle words; its warps
 // each sum a strided subset of the partials with independent loads, and the
 // warp sums are added in a fixed order, so D is an exact integer result
 // independent of scheduling.  The kernel writes both halves of the symmetric D
@@ -31,18 +31,15 @@ constexpr int kImgThreads = 1024;
 
 template <int EP>
 __global__ void __launch_bounds__(kRedThreads)
-cooc_reduce_kernel(const uint32_t *__restrict__ partials, int P1, const int *__restrict__ n_acc, int E,
-                   int *__restrict__ D, int *__restrict__ counts, unsigned char *__restrict__ bimg,
+cooc_reduce_kernel(const uint32_t *__restrict__ partials, int P1, int E, int *__restrict__ D, int *__restrict__ counts, unsigned char *__restrict__ bimg,
                    int big, long long *__restrict__ origin_do, long long r_base, int r_mult) {
     constexpr int kWords = tri_words(EP);
     __shared__ uint32_t s_sum[kRedWarps][33];
-    __shared__ int s_n[EP];  // the counts n_a, read once per CTA while the partials load
     const int e = threadIdx.x & 31, wp = threadIdx.x >> 5;
     const int word = blockIdx.x * 32 + e;
     const int layer = blockIdx.y;
     pdl_wait();
     pdl_trigger();
-    if ((int)threadIdx.x < E) s_n[threadIdx.x] = n_acc[(size_t)layer * E + threadIdx.x];
     uint32_t acc = 0u;
     const uint32_t *base = partials + (size_t)layer * P1 * kWords + word;
     for (int p0 = wp; p0 < P1; p0 += kRedLoads * kRedWarps) {
@@ -83,17 +80,18 @@ cooc_reduce_kernel(const uint32_t *__restrict__ partials, int P1, const int *__r
                 put_pieces(img, EP, b, a, 0, 0);
             }
         } else if (a == b) {
+            const int n = (int)(c >> 1);
             Dl[a * E + a] = 0;
-            counts[(size_t)layer * E + a] = (int)c;
+            counts[(size_t)layer * E + a] = n;
             // R_a = (E - 2k) n_a + T k (every row of the co-occurrence sums to k n_a)
-            const long long r = r_base + (long long)r_mult * (long long)c;
+            const long long r = r_base + (long long)r_mult * (long long)n;
             if (img) {
                 reinterpret_cast<float *>(img + bimg_r_offset(EP))[a] = (float)r;
                 if (big) put_pieces(img, EP, a, a, -32768, 0);
                 else put_dprime(img, EP, a, a, true, (int)r);
             }
         } else {
-            const int d = s_n[a] + s_n[b] - 2 * (int)c;
+            const int d = (int)c;
             Dl[a * E + b] = d;
             Dl[b * E + a] = d;
             if (img) {
@@ -112,8 +110,8 @@ cooc_reduce_kernel(const uint32_t *__restrict__ partials, int P1, const int *__r
 }
 
 template <int EP>
-cudaError_t run_reduce(const uint32_t *partials, int P1, const int *n_acc, const Problem &p, int *D,
-                       int *counts, unsigned char *bimg, bool big, long long *origin_do, cudaStream_t s) {
+cudaError_t run_reduce(const uint32_t *partials, int P1, const Problem &p, int *D, int *counts,
+                       unsigned char *bimg, bool big, long long *origin_do, cudaStream_t s) {
     constexpr int kWords = tri_words(EP);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((kWords + 31) / 32, (unsigned)p.L);
@@ -126,7 +124,7 @@ cudaError_t run_reduce(const uint32_t *partials, int P1, const int *n_acc, const
     cfg.numAttrs = 1;
     const long long r_base = p.T * (long long)p.k;
     const int r_mult = p.E - 2 * p.k;
-    return cudaLaunchKernelEx(&cfg, cooc_reduce_kernel<EP>, partials, P1, n_acc, p.E, D, counts, bimg,
+    return cudaLaunchKernelEx(&cfg, cooc_reduce_kernel<EP>, partials, P1, p.E, D, counts, bimg,
                               (int)big, origin_do, r_base, r_mult);
 }
 
@@ -219,19 +217,19 @@ dprime_image_kernel(const int *__restrict__ D, int E, int EP, unsigned char *__r
 
 }  // namespace
 
-cudaError_t launch_cooc_reduce(const uint32_t *partials, int P1, const int *n_acc, const Problem &p,
+cudaError_t launch_cooc_reduce(const uint32_t *partials, int P1, const Problem &p,
                                int *D, int *counts, unsigned char *bimg, bool big,
                                long long *origin_do, cudaStream_t s) {
     if (!cooc_sizes_ok(p.E, p.k) || (bimg && !bimg_sizes_ok(p.E, p.k))) return cudaErrorInvalidValue;
     switch (cooc_width(p.E)) {
-        case 32: return run_reduce<32>(partials, P1, n_acc, p, D, counts, bimg, big, origin_do, s);
-        case 64: return run_reduce<64>(partials, P1, n_acc, p, D, counts, bimg, big, origin_do, s);
-        case 96: return run_reduce<96>(partials, P1, n_acc, p, D, counts, bimg, big, origin_do, s);
-        case 128: return run_reduce<128>(partials, P1, n_acc, p, D, counts, bimg, big, origin_do, s);
-        case 160: return run_reduce<160>(partials, P1, n_acc, p, D, counts, bimg, big, origin_do, s);
-        case 192: return run_reduce<192>(partials, P1, n_acc, p, D, counts, bimg, big, origin_do, s);
-        case 224: return run_reduce<224>(partials, P1, n_acc, p, D, counts, bimg, big, origin_do, s);
-        default: return run_reduce<256>(partials, P1, n_acc, p, D, counts, bimg, big, origin_do, s);
+        case 32: return run_reduce<32>(partials, P1, p, D, counts, bimg, big, origin_do, s);
+        case 64: return run_reduce<64>(partials, P1, p, D, counts, bimg, big, origin_do, s);
+        case 96: return run_reduce<96>(partials, P1, p, D, counts, bimg, big, origin_do, s);
+        case 128: return run_reduce<128>(partials, P1, p, D, counts, bimg, big, origin_do, s);
+        case 160: return run_reduce<160>(partials, P1, p, D, counts, bimg, big, origin_do, s);
+        case 192: return run_reduce<192>(partials, P1, p, D, counts, bimg, big, origin_do, s);
+        case 224: return run_reduce<224>(partials, P1, p, D, counts, bimg, big, origin_do, s);
+        default: return run_reduce<256>(partials, P1, p, D, counts, bimg, big, origin_do, s);
     }
 }
 

@@ -67,16 +67,14 @@ struct ZeroSpans {
 //   done            [L] int, per-problem count of finished loss CTAs
 //   partials        [L][max CTAs per problem] fp64 sums of A_t
 //   idx             [L][T][k] uint8, the selected experts of every token
-//   cooc_parts      [L][P1][triangle words] uint32, per-CTA co-occurrence counts
-//   n_acc           [L][E] int32, counts summed by the signatures CTAs (kept at
-//                   zero between calls: the loss kernel clears it after use)
+//   cooc_parts      [L][P1][triangle words] uint32, per-CTA distances
 //   bimg            [L][bimg_bytes(EP)], the fp16 image of D' (E <= 128)
 //   img_ok          [L] int32, 1 where the image of a given (summed) D is exact
 //   route_base      route_scratch_ints int32, scratch of the dispatch order
 struct WsLayout {
-    size_t done, partials, idx, cooc_parts, n_acc, bimg, img_ok, route_base, total;
+    size_t done, partials, idx, cooc_parts, bimg, img_ok, route_base, total;
     int max_parts;  // partial slots per problem
-    bool cooc;      // the layout has cooc_parts and n_acc
+    bool cooc;      // the layout has cooc_parts
     bool image;     // ... and bimg
 };
 // Signatures CTAs per problem on the fast path: min(SMs, kMaxSigCtas) / L.
@@ -112,9 +110,9 @@ cudaError_t launch_hamming(const uint32_t *bits, const Problem &p, int *D, cudaS
 // 16-byte aligned logits).  counts: zero on entry; null: not counted.  idx
 // (may be null, E <= 256): the chosen experts of every token, one byte each.
 // zero: ranges cleared for the kernels after it.  status (may be null): the
-// device status word.  cooc (E <= 256, may be null): the per-CTA co-occurrence
-// triangles, sig_ctas_per_problem of them per problem; counts is then the
-// accumulator that the reduction reads.
+// device status word.  cooc (E <= 256, may be null): the per-CTA triangles,
+// sig_ctas_per_problem of them per problem (counts is then not written: the
+// reduction does).
 struct SelectOut {
     uint32_t *bits;
     int *counts;
@@ -145,12 +143,11 @@ cudaError_t launch_origin_do(const int *D, const Problem &p, long long *origin_d
 cudaError_t launch_offdiag_variance(const long long *origin_do, const Problem &p, double *var,
                                     cudaStream_t s);
 // Generic loss (any E, k).  counts (may be null): n_i of the same tokens, D being
-// their own matrix; n_zero ([L][E], may be null) is cleared.
+// their own matrix.
 cudaError_t launch_loss(const float *logits, const uint32_t *bits, const int *D,
                         const Problem &p, int gate, float d_scale, float grad_scale,
                         float *loss, long long *origin_do, float *dlogits, int *status,
-                        double *partials, cudaStream_t s, const int *counts = nullptr,
-                        int *n_zero = nullptr);
+                        double *partials, cudaStream_t s, const int *counts = nullptr);
 
 // Dispatch order of the routed (token, choice) pairs from the signatures and
 // the chosen ids alone: offsets [L][E+1], rows [L][T k], pos [L][T][k] (each
@@ -164,32 +161,27 @@ cudaError_t launch_route_backward(const float *z, const int32_t *ids, const floa
                                   int32_t E, int32_t k, int32_t gate, int32_t accumulate,
                                   float *dz, int32_t *status_flags, cudaStream_t s);
 
-// n_zero (may be null): an [L][E] accumulator cleared once the kernels before
-// these have finished (the scan kernel does it after its dependency wait).
 // counts_out (may be null): n_e = |F_e| from the scan's popcounts.
 cudaError_t launch_route_dispatch(const uint32_t *bits, const int *ids, const Problem &p,
                                   int *offsets, int *rows, int *pos, int *scratch,
-                                  cudaStream_t s, int *n_zero = nullptr,
-                                  int *counts_out = nullptr);
+                                  cudaStream_t s, int *counts_out = nullptr);
 // Router-side fusion (E = 128, k in {1,2,4,8}, H a multiple of 64, 16-byte
 // aligned X, W and logits): logits = X W^T on the tensor cores with the
 // fused path's signature step in the epilogue (bits, selected indices,
-// per-CTA co-occurrence triangles, counts accumulated into `counts`).
+// per-CTA triangles).
 bool router_supported(const Problem &p, int H, const void *X, const void *Wr, const float *logits);
 int router_ctas_per_problem(const Problem &p);
 cudaError_t launch_router_signatures(const void *X, const void *Wr, int H, float *logits,
-                                     const Problem &p, uint32_t *bits, int *counts, uint8_t *idx,
-                                     uint32_t *cooc, const ZeroSpans &zero, int *status,
-                                     cudaStream_t s);
+                                     const Problem &p, uint32_t *bits, uint8_t *idx, uint32_t *cooc,
+                                     const ZeroSpans &zero, int *status, cudaStream_t s);
 bool loss_fast_supported(const Problem &p, const float *logits, const int *D, const float *dlogits);
 // The E = 256 variant: counts given (D of the same tokens), T < 2^24.
 bool loss_fast256_supported(const Problem &p, const float *logits, const int *D,
                             const float *dlogits);
 cudaError_t launch_idx_from_bits(const uint32_t *bits, const Problem &p, uint8_t *idx, int *zero_ptr,
                                  int zero_n, cudaStream_t s);
-// counts: when given, R_i = (E - 2k) n_i + T k (D local to these tokens) and
-// n_zero ([L][E], may be null) is cleared once D is read; otherwise R_i is a
-// column sum of D.
+// counts: when given, R_i = (E - 2k) n_i + T k (D local to these tokens);
+// otherwise R_i is a column sum of D.
 // Tensor-core loss path (loss_mma.cuh).  bimg: the image of D' written by
 // launch_cooc_reduce for these tokens (marker diagonal where loss_mma_big), or
 // by launch_dprime_image for a given matrix D (where img_ok is 0, D is read
@@ -202,18 +194,21 @@ bool loss_mma_route_grad(const Problem &p, int gate, const int *ids, const float
 // idx (may be null; k in {1, 2, 4, 8}, E in {32, 64, 128}; needed for the routing
 // gradient): the chosen experts of every token, as the selection wrote them.
 cudaError_t launch_loss_mma(const float *logits, const uint32_t *bits, const uint8_t *idx,
-                            const unsigned char *bimg, int *n_zero, const Problem &p, int gate, float d_scale, float grad_scale,
+                            const unsigned char *bimg, const Problem &p, int gate, float d_scale, float grad_scale,
                             float *loss, float *dlogits, double *partials, int *done, int *status,
                             int *status_out, cudaStream_t s, const int *rg_ids = nullptr,
                             const float *rg_g = nullptr, const int *img_ok = nullptr,
                             const int *D = nullptr);
 cudaError_t launch_loss_fast(const float *logits, const uint8_t *idx, const int *D,
-                             const int *counts, int *n_zero, const Problem &p, int gate,
+                             const int *counts, const Problem &p, int gate,
                              float d_scale, float grad_scale, float *loss, long long *origin_do,
                              float *dlogits, double *partials, int *done, int *status,
                              int *status_out, cudaStream_t s);
 
-// Co-occurrence counts c_ab (a <= b) of one CTA are kept as a triangle in
+// What a selection CTA leaves of its tokens for the reduction is a triangle of
+// words d_ab = n_a + n_b - 2 c_ab (a < b; c_ab the tokens that chose both) and
+// d_aa = 2 n_a: distances add up over CTAs as the counts do, so that nothing else
+// has to be summed beside them or cleared before.  It is kept in
 // chunks of four columns: chunk c = b / 4 holds rows 0 .. 4c + 3, four words
 // each, so that the rows of a chunk are consecutive (a warp that holds a row
 // per lane stores 512 contiguous bytes).  Word of (a, b): tri_chunk(b / 4) +
@@ -262,7 +257,7 @@ __device__ __forceinline__ void put_dprime(unsigned char *img, int EP, int n, in
     put_pieces(img, EP, n, k, h, l);
 }
 
-// Whether the selection kernel can leave co-occurrence counts, the width of
+// Whether the selection kernel can leave the triangles of distances, the width of
 // its triangles and their words.
 inline bool cooc_sizes_ok(int E, int k) { return E % 4 == 0 && E <= 256 && k <= 16; }
 inline int cooc_width(int E) { return (E + 31) / 32 * 32; }
@@ -270,7 +265,7 @@ inline size_t cooc_partial_words(int E) { return (size_t)tri_words(cooc_width(E)
 // bimg ([L][bimg_bytes(EP)], E <= 128, may be null): the fp16 image of D' for
 // the tensor-core loss kernel, written alongside D (big: the marker diagonal).  origin_do (may be
 // null) must be zero on entry: sum_{a != b} D_ab^2 is added to it.
-cudaError_t launch_cooc_reduce(const uint32_t *partials, int P1, const int *n_acc, const Problem &p,
+cudaError_t launch_cooc_reduce(const uint32_t *partials, int P1, const Problem &p,
                                int *D, int *counts, unsigned char *bimg, bool big,
                                long long *origin_do, cudaStream_t s);
 // The image of D' from a given [L][E][E] matrix D (16-byte aligned; the split

@@ -217,15 +217,12 @@ loss_generic_kernel(const float *__restrict__ logits, const uint32_t *__restrict
 
 // loss[l] = d_scale/(m^2 k) * sum of the partials in block order.
 __global__ void __launch_bounds__(256)
-loss_finalize_kernel(const double *__restrict__ partials, int P, int E, double scale,
-                     float *__restrict__ loss, int *__restrict__ n_zero) {
+loss_finalize_kernel(const double *__restrict__ partials, int P, double scale,
+                     float *__restrict__ loss) {
     __shared__ double s_dred[256];
     const int layer = blockIdx.x;
     const double s = block_sum_fixed(partials + (int64_t)layer * P, P, s_dred, 256);
     if (threadIdx.x == 0) loss[layer] = (float)(s * scale);
-    // the counts accumulator has been read: cleared for the next call
-    if (n_zero)
-        for (int i = threadIdx.x; i < E; i += blockDim.x) n_zero[(int64_t)layer * E + i] = 0;
 }
 
 // origin_do += sum_{i != j} D_ij^2 over kOriginRows rows of one problem (Eq.
@@ -341,8 +338,7 @@ WsLayout ws_layout(const Problem &p, bool wide) {
                                                   (size_t)max_sig_ctas_per_problem(p) *
                                                   cooc_partial_words(p.E)
                                             : 0;
-    w.n_acc = up(w.cooc_parts + parts);
-    w.bimg = up(w.n_acc + (w.cooc ? sizeof(int) * (size_t)p.L * p.E : 0));
+    w.bimg = up(w.cooc_parts + parts);
     // the dispatch order of a routed call may run beside the loss kernel: its
     // scratch has a region of its own
     w.img_ok = up(w.bimg + (w.image ? (size_t)bimg_bytes(cooc_width(p.E)) * (size_t)p.L : 0));
@@ -360,7 +356,7 @@ int max_sig_ctas_per_problem(const Problem &p) {
 cudaError_t launch_loss(const float *logits, const uint32_t *bits, const int *D, const Problem &p,
                         int gate, float d_scale, float grad_scale, float *loss,
                         long long *origin_do, float *dlogits, int *status, double *partials,
-                        cudaStream_t s, const int *counts, int *n_zero) {
+                        cudaStream_t s, const int *counts) {
     const double norm = 1.0 / ((double)p.T * (double)p.T * (double)p.k);
     const GenericArgs a = {logits, bits, D, counts, (float)((double)grad_scale * (double)d_scale * norm),
                            dlogits, partials, ws_layout(p, false).max_parts, status};
@@ -374,7 +370,7 @@ cudaError_t launch_loss(const float *logits, const uint32_t *bits, const int *D,
     else if (r <= 16) e = dispatch_gate<16>(a, p, gate, &P, s);
     else e = dispatch_gate<32>(a, p, gate, &P, s);
     if (e != cudaSuccess) return e;
-    loss_finalize_kernel<<<p.L, 256, 0, s>>>(partials, P, p.E, (double)d_scale * norm, loss, n_zero);
+    loss_finalize_kernel<<<p.L, 256, 0, s>>>(partials, P, (double)d_scale * norm, loss);
     e = cudaGetLastError();
     if (e == cudaSuccess && origin_do) e = launch_origin_do(D, p, origin_do, s);
     return e;

@@ -100,7 +100,6 @@ struct LossArgs {
     const uint8_t *idx;
     const int *D;        // [L][E][E], symmetric
     const int *counts;   // fused path: n_i [L][E] of the same tokens (else null)
-    int *n_zero;         // fused path: accumulator [L][E] to clear after use (or null)
     int64_t T;
     int k;
     int tokens_per_cta;
@@ -210,7 +209,6 @@ loss_fast_kernel(const LossArgs a) {
             if (r > INT_MAX || r < 0) atomicOr(a.status, kDevOverflow);
             if (kPlanes) s_rp[i] = (int)r;
             else sD[i * E + i] = -(int)r;
-            if (a.n_zero && blockIdx.x == 0) a.n_zero[(int64_t)layer * E + i] = 0;
         }
     } else {
         // R_i = sum_j D_ji (D symmetric): kPer threads per column, four chains each
@@ -600,7 +598,7 @@ cudaError_t launch_idx_from_bits(const uint32_t *bits, const Problem &p, uint8_t
 }
 
 cudaError_t launch_loss_fast(const float *logits, const uint8_t *idx, const int *D,
-                             const int *counts, int *n_zero, const Problem &p, int gate,
+                             const int *counts, const Problem &p, int gate,
                              float d_scale, float grad_scale, float *loss, long long *origin_do,
                              float *dlogits, double *partials, int *done, int *status,
                              int *status_out, cudaStream_t s) {
@@ -612,7 +610,6 @@ cudaError_t launch_loss_fast(const float *logits, const uint8_t *idx, const int 
     args.idx = idx;
     args.D = D;
     args.counts = counts;
-    args.n_zero = n_zero;
     args.T = p.T;
     args.k = p.k;
     args.tokens_per_cta = tpc;

@@ -55,7 +55,7 @@ bool loss_mma_route_grad(const Problem &p, int gate, const int *ids, const float
 }
 
 cudaError_t launch_loss_mma(const float *logits, const uint32_t *bits, const uint8_t *idx,
-                            const unsigned char *bimg, int *n_zero, const Problem &p, int gate, float d_scale, float grad_scale,
+                            const unsigned char *bimg, const Problem &p, int gate, float d_scale, float grad_scale,
                             float *loss, float *dlogits, double *partials, int *done, int *status,
                             int *status_out, cudaStream_t s, const int *rg_ids, const float *rg_g,
                             const int *img_ok, const int *D) {
@@ -77,7 +77,6 @@ cudaError_t launch_loss_mma(const float *logits, const uint32_t *bits, const uin
     args.idx = idx;
     args.k = p.k;
     args.bimg = bimg;
-    args.n_zero = n_zero;
     args.T = p.T;
     args.W = p.W;
     args.E = p.E;

@@ -25,9 +25,10 @@
 //            warps that end the kernel) and the signature words run on that
 //            tile.  The co-occurrence counts go into a shared triangle
 //            of 16-bit counters (two per word: the CTA's range is below 65536
-//            tokens), written out unpacked at the end; for longer ranges they
+//            tokens); for longer ranges they
 //            go straight to the CTA's triangle in global memory as L2
-//            reductions.
+//            reductions.  At the end the triangle goes out as distances
+//            n_a + n_b - 2 c_ab.
 
 #include "sig_fast.cuh"
 #include "topk_net.cuh"
@@ -51,7 +52,8 @@ constexpr int kRTriWords = tri_words(kRE);
 
 constexpr size_t kROffZ = (size_t)kRStages * kRStageBytes;
 constexpr size_t kROffColoff = kROffZ + (size_t)kREpiWarps * kRZTileBytes;
-constexpr size_t kROffTri = kROffColoff + (size_t)kRE * 4;          // packed 16-bit counters
+constexpr size_t kROffN = kROffColoff + (size_t)kRE * 4;            // counts n_a
+constexpr size_t kROffTri = kROffN + (size_t)kRE * 4;               // packed 16-bit counters
 constexpr size_t kROffBars = kROffTri + (size_t)(kRTriWords / 2) * 4;
 constexpr size_t kRNumBars = 2 * kRStages + 4;
 constexpr size_t kROffScal = kROffBars + kRNumBars * 8;
@@ -64,7 +66,6 @@ struct RouterArgs {
     uint32_t *bits;
     uint8_t *idx;
     uint32_t *cooc;
-    int *counts;
     ZeroSpans zero;
     int *status;
 };
@@ -110,6 +111,7 @@ router_sig_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constan
     unsigned char *ring = smem;
     unsigned char *ztiles = smem + kROffZ;
     int *s_coloff = reinterpret_cast<int *>(smem + kROffColoff);
+    uint32_t *s_n = reinterpret_cast<uint32_t *>(smem + kROffN);
     uint32_t *s_tri = reinterpret_cast<uint32_t *>(smem + kROffTri);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kROffBars);
     uint64_t *full = bars, *empty = bars + kRStages;
@@ -124,11 +126,14 @@ router_sig_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constan
     // this CTA's signature words [wb, we): an even split of the problem's W words
     const int64_t wb = (int64_t)blockIdx.x * a.W / gridDim.x;
     const int64_t we = (int64_t)(blockIdx.x + 1) * a.W / gridDim.x;
-    // this CTA's co-occurrence triangle (the reduction kernel's input)
+    // this CTA's triangle (the reduction kernel's input)
     uint32_t *tri = a.cooc + ((size_t)layer * gridDim.x + blockIdx.x) * (size_t)kRTriWords;
     // Shared-memory and TMEM set-up touch no global memory: they overlap the
     // end of the previous kernel on the stream.
-    for (int e = threadIdx.x; e < kRE; e += kRThreads) s_coloff[e] = tri_chunk(e >> 2) + (e & 3);
+    for (int e = threadIdx.x; e < kRE; e += kRThreads) {
+        s_coloff[e] = tri_chunk(e >> 2) + (e & 3);
+        s_n[e] = 0u;
+    }
     if (a.packed)
         for (int i = threadIdx.x; i < kRTriWords / 2; i += kRThreads) s_tri[i] = 0u;
     if (threadIdx.x == 0) {
@@ -305,22 +310,33 @@ router_sig_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constan
             }
         }
         if (lane == 0) bulk_wait_all<0>();  // the last stores are complete before exit
-        // counts n_a: on the triangle's diagonal and into the problem's totals
+        // once all epilogue warps have counted: the triangle out as distances
+        // n_a + n_b - 2 c_ab (2 n_a on the diagonal), a warp per chunk of four columns
 #pragma unroll
         for (int r = 0; r < kRE / 32; ++r)
-            if (cnt[r]) {
-                const int e = 32 * r + lane;
-                const int wi = s_coloff[e] + 4 * e;
-                if (a.packed) atomicAdd(&s_tri[wi >> 1], cnt[r] << (16 * (wi & 1)));
-                else atomicAdd(&tri[wi], cnt[r]);
-                atomicAdd(&a.counts[layer * kRE + e], (int)cnt[r]);
-            }
-        if (a.packed) {
-            // all epilogue warps have counted: the triangle out, unpacked
-            asm volatile("bar.sync 1, %0;" ::"n"(kREpiWarps * 32) : "memory");
-            for (int q = threadIdx.x - 64; q < kRTriWords / 2; q += kREpiWarps * 32) {
-                const uint32_t v = s_tri[q];
-                reinterpret_cast<uint2 *>(tri)[q] = make_uint2(v & 0xFFFFu, v >> 16);
+            if (cnt[r]) atomicAdd(&s_n[32 * r + lane], cnt[r]);
+        if (!a.packed) __threadfence();
+        asm volatile("bar.sync 1, %0;" ::"n"(kREpiWarps * 32) : "memory");
+        uint32_t na[kRE / 32];
+#pragma unroll
+        for (int r = 0; r < kRE / 32; ++r) na[r] = s_n[32 * r + lane];
+#pragma unroll
+        for (int v = 0; v < kRE / 16; ++v) {
+            const int c = kREpiWarps * v + ew, q0 = tri_chunk(c) / 4 + lane;
+            const uint4 nb = reinterpret_cast<const uint4 *>(s_n)[c];
+#pragma unroll
+            for (int r = 0; r <= v / 2; ++r) {
+                if (r == v / 2 && lane >= 4 * (c & 7) + 4) continue;
+                uint4 x;
+                if (a.packed) {
+                    const uint2 h = reinterpret_cast<const uint2 *>(s_tri)[q0 + 32 * r];
+                    x = make_uint4(h.x & 0xFFFFu, h.x >> 16, h.y & 0xFFFFu, h.y >> 16);
+                } else {
+                    x = __ldcg(reinterpret_cast<const uint4 *>(tri) + q0 + 32 * r);
+                }
+                reinterpret_cast<uint4 *>(tri)[q0 + 32 * r] =
+                    make_uint4(na[r] + nb.x - 2 * x.x, na[r] + nb.y - 2 * x.y, na[r] + nb.z - 2 * x.z,
+                               na[r] + nb.w - 2 * x.w);
             }
         }
     }
@@ -378,9 +394,8 @@ int router_ctas_per_problem(const Problem &p) {
 }
 
 cudaError_t launch_router_signatures(const void *X, const void *Wr, int H, float *logits,
-                                     const Problem &p, uint32_t *bits, int *counts, uint8_t *idx,
-                                     uint32_t *cooc, const ZeroSpans &zero, int *status,
-                                     cudaStream_t s) {
+                                     const Problem &p, uint32_t *bits, uint8_t *idx, uint32_t *cooc,
+                                     const ZeroSpans &zero, int *status, cudaStream_t s) {
     CUtensorMap xm, wm, zm;
     if (!encode_tensor_map_3d_bf16(&xm, X, (uint64_t)p.L, (uint64_t)p.T, (uint64_t)H, kRSlice, 32) ||
         !encode_tensor_map_3d_bf16(&wm, Wr, (uint64_t)p.L, (uint64_t)kRE, (uint64_t)H, kRSlice, kRE) ||
@@ -397,7 +412,6 @@ cudaError_t launch_router_signatures(const void *X, const void *Wr, int H, float
     a.bits = bits;
     a.idx = idx;
     a.cooc = cooc;
-    a.counts = counts;
     a.zero = zero;
     a.status = status;
     switch (p.k) {

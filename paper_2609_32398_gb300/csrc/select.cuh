@@ -26,7 +26,8 @@
 // (the tile's own slot holds them once the logits are read) and one thread
 // adds F^T F on the tensor cores into an accumulator that stays in TMEM for
 // the whole CTA: c_ab = sum_t f_at f_bt, exact (0/1 products, fp32 sums), in
-// place of k (k - 1) / 2 shared-memory atomics per token.
+// place of k (k - 1) / 2 shared-memory atomics per token.  At the end it goes
+// out as the CTA's triangle of distances n_a + n_b - 2 c_ab.
 // With routing outputs the lane also writes the chosen experts in selection
 // order and their re-normalized combine weights (Sec. 3.1.1).
 #pragma once
@@ -91,8 +92,8 @@ struct SelArgs {
     int whole;        // E a multiple of 32: the tensor map is [E / 32][L T][32]
     SelLayout lay;
     uint32_t *bits;
-    int *counts;      // kCooc: the counts accumulator; else the counts (zero on entry) or null
-    uint32_t *cooc;   // kCooc: per-CTA triangles of EP = 32 nb experts
+    int *counts;      // not kCooc: the counts (zero on entry) or null
+    uint32_t *cooc;   // kCooc: per-CTA triangles of distances of EP = 32 nb experts
     ZeroSpans zero;
     int *status;      // may be null
     uint8_t *idx;     // may be null: the chosen experts of every token, one byte each
@@ -502,39 +503,55 @@ select_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ 
     __syncthreads();
     tc_fence_after();
     if (kCooc) {
-        // this CTA's triangle of c_ab, TMEM -> registers -> global, for the
-        // reduction kernel; its diagonal, the counts n_a, is added to the
-        // layer's totals
+        // this CTA's triangle, TMEM -> registers -> global, for the reduction
+        // kernel: first the counts n_a = c_aa, then n_a + n_b - 2 c_ab (2 n_a on
+        // the diagonal)
         const int EP = 32 * nb;
         const int words = tri_words(EP);
         uint32_t *tri = a.cooc + ((size_t)layer * gridDim.x + blockIdx.x) * (size_t)words;
-        if (n == 0 || *s_abort) {
+        const bool any = n > 0 && !*s_abort;
+        const uint32_t tmem = any ? *s_tmem : 0u;
+        const int quad = warp & 3;
+        const uint32_t tquad = tmem + ((uint32_t)(32 * quad) << 16);
+        auto block_col = [](int blk, int cb) { return (uint32_t)(blk ? 256 + 32 * (cb - 4) : 32 * cb); };
+        uint32_t r[32];
+        if (any && warp < 4) {
+            for (int cb = quad; cb < nb; cb += 4) {  // the diagonal block of rows 32 cb ..
+                tmem_ld32(tquad + block_col(cb >> 2, cb), r);
+                tmem_wait_ld();
+                uint32_t na = r[0];
+#pragma unroll
+                for (int c = 1; c < 32; ++c) na = lane == c ? r[c] : na;
+                s_cnt[32 * cb + lane] = (int)(__uint_as_float(na) * 0.25f);
+            }
+        }
+        __syncthreads();
+        if (!any) {
             for (int i = threadIdx.x; i < words; i += blockDim.x) tri[i] = 0u;
         } else if (warp < (consumers & ~3)) {
-            const uint32_t tmem = *s_tmem;
-            const int quad = warp & 3, per = consumers >> 2;
+            const int per = consumers >> 2;
             const int nblk = nb <= 4 ? 1 : 2;
             for (int item = warp >> 2; item < nblk * nb; item += per) {
                 const int blk = item / nb, cb = item - blk * nb;
                 const int row0 = 128 * blk + 32 * quad;
                 if (row0 >= EP || 32 * cb + 31 < row0) continue;
                 const int row = row0 + lane;
-                uint32_t r[32];
-                const uint32_t col = blk ? 256 + 32 * (cb - 4) : 32 * cb;
-                tmem_ld32(tmem + ((uint32_t)(32 * quad) << 16) + col, r);
+                tmem_ld32(tquad + block_col(blk, cb), r);
                 tmem_wait_ld();
+                const int na = s_cnt[row];
 #pragma unroll
-                for (int c = 0; c < 32; ++c) r[c] = (uint32_t)(__uint_as_float(r[c]) * 0.25f);
+                for (int c = 0; c < 8; ++c) {
+                    const int4 nc = *reinterpret_cast<const int4 *>(s_cnt + 32 * cb + 4 * c);
+                    const int n4[4] = {nc.x, nc.y, nc.z, nc.w};
 #pragma unroll
-                for (int c = 0; c < 8; ++c)
+                    for (int u = 0; u < 4; ++u) {
+                        // 2 c_ab (F holds 2 instead of 1: the accumulator is 4 c_ab)
+                        const int both = 32 * cb + 4 * c + u == row ? 0 : (int)(__uint_as_float(r[4 * c + u]) * 0.5f);
+                        r[4 * c + u] = (uint32_t)(na + n4[u] - both);
+                    }
                     if (32 * cb + 4 * c + 4 > row)
                         *reinterpret_cast<uint4 *>(tri + tri_chunk(8 * cb + c) + 4 * row) =
                             make_uint4(r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
-                if (32 * cb == row0) {  // the diagonal block
-                    uint32_t na = r[0];
-#pragma unroll
-                    for (int c = 1; c < 32; ++c) na = lane >= c ? r[c] : na;
-                    if (na && row < E) atomicAdd(&a.counts[layer * E + row], (int)na);
                 }
             }
         }

@@ -46,10 +46,10 @@ struct SigCfg {
     static constexpr int kSlots = (E == 128) ? 11 : 16;
     static constexpr int GS = (E >= 128) ? E / 16 : 4;  // experts per group
     static constexpr int NG = E / GS;                    // groups per row
-    // co-occurrence counters in the triangle of tri_chunk
+    // co-occurrence counters in the triangle of tri_chunk, then counts n_a
     static constexpr int kCoocWords = tri_words(E);
     static constexpr size_t kSmem = (size_t)kSlots * kTileBytes + 1024 + 2 * kSlots * 8 +
-                                    kSlots * 4 + 32 + (size_t)kCoocWords * 4 + E * 4 +
+                                    kSlots * 4 + 32 + (size_t)kCoocWords * 4 + 2 * E * 4 +
                                     (size_t)kConsumers * E * 4;
 };
 
@@ -198,9 +198,9 @@ __device__ __forceinline__ void sort_small(int (&so)[K]) {
     }
 }
 
-// c_ab += 1 for every pair a < b of one token's chosen experts, in a
-// shared-memory triangle whose column b starts at s_coloff[b] (the counts on
-// the diagonal come from the signature words).
+// -2 for every pair a < b of one token's chosen experts (-2 c_ab), in a
+// shared-memory triangle whose column b starts at s_coloff[b] (the counts n_a
+// come from the signature words).
 template <int K>
 __device__ __forceinline__ void cooc_add(uint32_t *s_cooc, const int *s_coloff, const int (&sel)[K]) {
     int so[K];
@@ -211,7 +211,7 @@ __device__ __forceinline__ void cooc_add(uint32_t *s_cooc, const int *s_coloff, 
     for (int q2 = 1; q2 < K; ++q2) {
         uint32_t *col = s_cooc + s_coloff[so[q2]];
 #pragma unroll
-        for (int q1 = 0; q1 < q2; ++q1) atomicAdd(col + 4 * so[q1], 1u);
+        for (int q1 = 0; q1 < q2; ++q1) atomicAdd(col + 4 * so[q1], 0u - 2u);
     }
 }
 
@@ -258,7 +258,8 @@ sig_fast_kernel(const __grid_constant__ CUtensorMap tmap, int64_t T, int64_t W,
     volatile int *s_abort = slot_round + C::kSlots;
     uint32_t *s_cooc = reinterpret_cast<uint32_t *>(
         smem_align<16>(reinterpret_cast<unsigned char *>(const_cast<int *>(s_abort + 1))));
-    int *s_coloff = reinterpret_cast<int *>(s_cooc + C::kCoocWords);
+    uint32_t *s_n = s_cooc + C::kCoocWords;  // [E]
+    int *s_coloff = reinterpret_cast<int *>(s_n + E);
     uint32_t *s_wsc = reinterpret_cast<uint32_t *>(s_coloff + E);  // [consumer warp][E]
 
     pdl_trigger();
@@ -275,7 +276,7 @@ sig_fast_kernel(const __grid_constant__ CUtensorMap tmap, int64_t T, int64_t W,
     // the end of the previous kernel on the stream.
     for (int i = threadIdx.x; i < kConsumers * E; i += blockDim.x) s_wsc[i] = 0u;
     if (kCooc) {
-        for (int i = threadIdx.x; i < C::kCoocWords; i += blockDim.x) s_cooc[i] = 0u;
+        for (int i = threadIdx.x; i < C::kCoocWords + E; i += blockDim.x) s_cooc[i] = 0u;  // and s_n
         for (int a = threadIdx.x; a < E; a += blockDim.x) s_coloff[a] = tri_chunk(a >> 2) + (a & 3);
     }
     if (threadIdx.x == 0) {
@@ -376,24 +377,34 @@ sig_fast_kernel(const __grid_constant__ CUtensorMap tmap, int64_t T, int64_t W,
         for (int r = 0; r < R; ++r)
             if (cnt[r]) atomicAdd(&counts[layer * E + 32 * r + lane], (int)cnt[r]);
     }
-    if (kCooc) {  // counts n_a on the triangle's diagonal
+    if (kCooc) {
 #pragma unroll
         for (int r = 0; r < R; ++r)
-            if (cnt[r]) atomicAdd(&s_cooc[s_coloff[32 * r + lane] + 4 * (32 * r + lane)], cnt[r]);
-    }
-    if (kCooc) {
-        // all consumer warps have counted: store this CTA's triangle for the
-        // reduction kernel
+            if (cnt[r]) atomicAdd(&s_n[32 * r + lane], cnt[r]);
+        // all consumer warps have counted: this CTA's triangle of distances
+        // n_a + n_b - 2 c_ab (2 n_a on the diagonal) for the reduction kernel.  A
+        // warp takes chunks 8 v + warp of four columns, 32 rows at a time (all of
+        // it unrolled: 30.4 against 31.0 us of the E = 128, T = 65536 step with
+        // a loop over the rows of each chunk)
+        static_assert(kConsumers == 8, "chunks per 32 columns");
         asm volatile("bar.sync 1, %0;" ::"n"(kConsumers * 32) : "memory");
         uint4 *dst = reinterpret_cast<uint4 *>(cooc + ((size_t)layer * gridDim.x + blockIdx.x) *
                                                           (size_t)C::kCoocWords);
         const uint4 *src = reinterpret_cast<const uint4 *>(s_cooc);
-        for (int i = threadIdx.x; i < C::kCoocWords / 4; i += kConsumers * 32) dst[i] = src[i];
-        // the diagonal holds this CTA's counts n_a: add them to the layer's totals
-        // (counts points at the workspace accumulator on this path)
-        for (int a = threadIdx.x; a < E; a += kConsumers * 32) {
-            const uint32_t na = s_cooc[s_coloff[a] + 4 * a];
-            if (na) atomicAdd(&counts[layer * E + a], (int)na);
+        uint32_t na[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) na[r] = s_n[32 * r + lane];
+#pragma unroll
+        for (int v = 0; v < R; ++v) {
+            const int c = 8 * v + warp, q0 = tri_chunk(c) / 4 + lane;
+            const uint4 nb = reinterpret_cast<const uint4 *>(s_n)[c];
+#pragma unroll
+            for (int r = 0; r <= v; ++r) {
+                if (r == v && lane >= 4 * warp + 4) continue;
+                const uint4 x = src[q0 + 32 * r];
+                dst[q0 + 32 * r] = make_uint4(x.x + na[r] + nb.x, x.y + na[r] + nb.y, x.z + na[r] + nb.z,
+                                              x.w + na[r] + nb.w);
+            }
         }
     }
 }

@@ -122,17 +122,12 @@ extern "C" do_status do_forward_backward_static(const float *logits, int64_t T, 
     do_status st = scratch_on_current_device(&ws);
     if (st != DO_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // What must be zero when a call starts: the status word and the done
-    // counters (the first 256-byte-aligned span) and the counts accumulator
-    // [n_acc, bimg).  The kernels leave them zero after a complete call;
-    // clearing them here also recovers from a call that gave up on a wait.
-    // Everything else in the array is written before it is read (the image
-    // of D' at bimg by the reduction kernel, every entry of it).
-    const dol::WsLayout w = dol::ws_layout_for(p, DO_STATIC_SCRATCH_BYTES, true);
+    // What must be zero when a call starts is the status word; clearing it here
+    // also recovers from a call that gave up on a wait.  Everything else in the
+    // array is written before it is read (the done counters by the selection
+    // kernel, the image of D' by the reduction kernel, every entry of it).
     char *base = static_cast<char *>(ws);
-    if (cudaMemsetAsync(base, 0, w.partials, s) != cudaSuccess) return DO_ERR_CUDA;
-    if (w.bimg > w.n_acc && cudaMemsetAsync(base + w.n_acc, 0, w.bimg - w.n_acc, s) != cudaSuccess)
-        return DO_ERR_CUDA;
+    if (cudaMemsetAsync(base, 0, dol::kWsHeader, s) != cudaSuccess) return DO_ERR_CUDA;
     st = do_forward_backward(logits, T, E, k, L, gate, grad_scale, bits, counts, D, loss, origin_do,
                              dlogits, ws, DO_STATIC_SCRATCH_BYTES, stream);
     if (st != DO_OK) return st;

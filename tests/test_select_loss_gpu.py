@@ -145,6 +145,34 @@ def test_low_logits(dl, T, E, k, shift):
     check_loss(z[0].numpy(), f, D, k, 0, float(loss[0]), dz[0], zmax=zmax)
 
 
+# one zeroed workspace for two shapes in turn, both orders, each also twice running:
+# nothing that a call leaves in it may reach the next one
+@pytest.mark.parametrize("one,two", [
+    ((1, 40000, 256, 8), (1, 1000, 256, 8)), ((1, 30000, 96, 6), (3, 700, 96, 6)),
+    ((1, 65536, 128, 8), (1, 9000, 64, 8)), ((2, 9000, 160, 3), (1, 500, 8, 2)), ((4, 3000, 32, 2), (1, 20000, 128, 5))])
+def test_workspace_of_two_shapes(dl, one, two):
+    n = max(int(dl.lib().do_routed_workspace_size(T, E, k, L)) for L, T, E, k in (one, two))
+    ws = torch.zeros(n, dtype=torch.uint8, device="cuda")
+
+    def run(shape, z, routed, ws=None):
+        out = dl.Buffers(*shape)
+        if ws is not None:
+            out.workspace = ws
+        if not routed:
+            return dl.forward_backward(z, shape[3], out=out)
+        dl.routed_forward(z, shape[3], out=out)
+        return dl.routed_backward(z, None, None, shape[3], out=out)
+
+    z = {s: workloads.random_logits(s[1], s[2], L=s[0], seed=s[2] + s[3]).cuda() for s in (one, two)}
+    want = {(s, r): run(s, z[s], r) for s in (one, two) for r in (False, True)}
+    for shape in (one, two, two, one, one):
+        for routed in (False, True):
+            out = run(shape, z[shape], routed, ws)
+            for name in ("counts", "D", "origin_do", "loss", "dlogits"):
+                assert torch.equal(getattr(out, name), getattr(want[shape, routed], name)), (shape, routed, name)
+    assert dl.device_status(ws) == 0
+
+
 # a given matrix: its image (the first problem), and one that no image holds (an
 # entry of 2^22, or a non-zero diagonal), gathered from D in the same launch.  A
 # non-zero diagonal, which no matrix of distances has, only at sizes of the
