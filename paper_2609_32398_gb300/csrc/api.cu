@@ -170,10 +170,10 @@ do_status do_loss_fwd_bwd(const float *logits, const uint32_t *bits, const int32
     if (!aligned(logits, 4) || !aligned(bits, 4) || !aligned(D, 4) || !aligned(loss, 4) ||
         (dlogits && !aligned(dlogits, 4)) || (origin_do && !aligned(origin_do, 8)))
         return DO_ERR_INVALID_ARG;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < dol::workspace_bytes_plain(p, false))
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < dol::workspace_bytes_plain(p))
         return DO_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
-    const dol::WsLayout w = dol::ws_layout_for(p, workspace_bytes, true);
+    const dol::WsLayout w = dol::ws_layout(p);
     char *ws = static_cast<char *>(workspace);
     int *done = reinterpret_cast<int *>(ws + w.done);
     int *status = reinterpret_cast<int *>(ws);
@@ -183,7 +183,7 @@ do_status do_loss_fwd_bwd(const float *logits, const uint32_t *bits, const int32
     cudaError_t e = cudaSuccess;
     const bool alu = dol::loss_fast_supported(p, logits, D, dlogits) && aligned(bits, 16);
     // (the fused call's kernel: the same results bit for bit)
-    if (w.image && dol::loss_mma_supported(p, logits, dlogits) && aligned(D, 16) &&
+    if (dol::loss_mma_supported(p, logits, dlogits) && aligned(D, 16) &&
         !(alu && dol::loss_alu_faster(p, gate))) {
         // the given matrix's image of D' and origin_do, then the tensor-core kernel
         unsigned char *bimg = reinterpret_cast<unsigned char *>(ws + w.bimg);
@@ -212,13 +212,15 @@ namespace {
 
 // Steps 1-3.  status_out (may be null): on the fused fast path the last loss
 // CTA ORs the device status word of this call into it (so that one copy
-// returns the loss and the status); *status_done tells whether it did.
+// returns the loss and the status); *status_done tells whether it did.  wide:
+// the workspace's layout.
 do_status forward_backward_impl(const float *logits, int64_t T, int32_t E, int32_t k, int32_t L,
                                 int32_t gate, float grad_scale, uint32_t *bits, int32_t *counts,
                                 int32_t *D, float *loss, int64_t *origin_do, float *dlogits,
                                 void *workspace, size_t workspace_bytes, void *stream,
                                 int *status_out, bool *status_done,
-                                const RouteArgs *ra = nullptr, const RouterIn *rin = nullptr) {
+                                const RouteArgs *ra = nullptr, const RouterIn *rin = nullptr,
+                                bool wide = true) {
     if (status_done) *status_done = false;
     Problem p;
     do_status st = check_sizes(T, E, k, L, &p);
@@ -231,10 +233,10 @@ do_status forward_backward_impl(const float *logits, int64_t T, int32_t E, int32
         (origin_do && !aligned(origin_do, 8)))
         return DO_ERR_INVALID_ARG;
     if (ra && (st = check_route(p, *ra)) != DO_OK) return st;
-    const size_t need = ra ? dol::workspace_bytes(p, false) : dol::workspace_bytes_plain(p, false);
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < need) return DO_ERR_WORKSPACE;
+    const dol::WsLayout w = dol::ws_layout(p, wide);
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < (ra ? w.total : w.route_base))
+        return DO_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
-    const dol::WsLayout w = dol::ws_layout_for(p, workspace_bytes, !ra);
     char *ws = static_cast<char *>(workspace);
     int *done = reinterpret_cast<int *>(ws + w.done);
     int *status = reinterpret_cast<int *>(ws);
@@ -315,16 +317,25 @@ do_status forward_backward_impl(const float *logits, int64_t T, int32_t E, int32
 
 }  // namespace
 
+do_status dol::forward_backward_plain(const float *logits, int64_t T, int32_t E, int32_t k, int32_t L,
+                                      int32_t gate, float grad_scale, uint32_t *bits, int32_t *counts,
+                                      int32_t *D, float *loss, int64_t *origin_do, float *dlogits,
+                                      void *workspace, size_t workspace_bytes, void *stream,
+                                      bool wide) {
+    NvtxRange nvtx("do_forward_backward");
+    return forward_backward_impl(logits, T, E, k, L, gate, grad_scale, bits, counts, D, loss,
+                                 origin_do, dlogits, workspace, workspace_bytes, stream, nullptr,
+                                 nullptr, nullptr, nullptr, wide);
+}
+
 extern "C" {
 
 do_status do_forward_backward(const float *logits, int64_t T, int32_t E, int32_t k, int32_t L,
                               int32_t gate, float grad_scale, uint32_t *bits, int32_t *counts,
                               int32_t *D, float *loss, int64_t *origin_do, float *dlogits,
                               void *workspace, size_t workspace_bytes, void *stream) {
-    NvtxRange nvtx("do_forward_backward");
-    return forward_backward_impl(logits, T, E, k, L, gate, grad_scale, bits, counts, D, loss,
-                                 origin_do, dlogits, workspace, workspace_bytes, stream, nullptr,
-                                 nullptr);
+    return dol::forward_backward_plain(logits, T, E, k, L, gate, grad_scale, bits, counts, D, loss,
+                                       origin_do, dlogits, workspace, workspace_bytes, stream, true);
 }
 
 do_status do_forward_backward_routed(const float *logits, int64_t T, int32_t E, int32_t k,
@@ -367,8 +378,8 @@ bool split_fast(const Problem &p, const float *logits, const uint32_t *bits, con
 
 // Whether the forward half writes the fp16 image of D' for the tensor-core
 // loss kernel (dlogits is not known there).
-bool split_mma(const Problem &p, const float *logits, const dol::WsLayout &w) {
-    return dol::select_supported(logits, p) && w.image && dol::loss_mma_supported(p, logits, nullptr);
+bool split_mma(const Problem &p, const float *logits) {
+    return dol::select_supported(logits, p) && dol::loss_mma_supported(p, logits, nullptr);
 }
 
 do_status do_routed_forward(const float *logits, int64_t T, int32_t E, int32_t k, int32_t L,
@@ -391,11 +402,11 @@ do_status do_routed_forward(const float *logits, int64_t T, int32_t E, int32_t k
     const RouteArgs ra = {expert_ids, combine, expert_offsets, dispatch_rows, dispatch_pos};
     if (routed && (st = check_route(p, ra)) != DO_OK) return st;
     if (!routed && (expert_offsets || dispatch_rows || dispatch_pos)) return DO_ERR_INVALID_ARG;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < dol::workspace_bytes(p, false))
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < dol::workspace_bytes(p))
         return DO_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
     char *ws = static_cast<char *>(workspace);
-    const dol::WsLayout w = dol::ws_layout_for(p, workspace_bytes, false);
+    const dol::WsLayout w = dol::ws_layout(p);
     int *rscratch = reinterpret_cast<int *>(ws + w.route_base);
     const dol::RouteOut route = {expert_ids, combine, gate};
     cudaError_t e = cudaSuccess;
@@ -405,7 +416,7 @@ do_status do_routed_forward(const float *logits, int64_t T, int32_t E, int32_t k
         const dol::ZeroSpans zero = {{done, reinterpret_cast<int *>(origin_do), nullptr},
                                      {(int64_t)p.L, origin_do ? 2 * (int64_t)p.L : 0, 0}};
         // what the backward half's loss kernel reads
-        unsigned char *bimg = split_mma(p, logits, w)
+        unsigned char *bimg = split_mma(p, logits)
                                   ? reinterpret_cast<unsigned char *>(ws + w.bimg) : nullptr;
         uint8_t *idx = dol::signatures_fast_supported(logits, p)
                            ? reinterpret_cast<uint8_t *>(ws + w.idx) : nullptr;
@@ -446,11 +457,11 @@ do_status do_routed_backward(const float *logits, int64_t T, int32_t E, int32_t 
         (rg && (!aligned(expert_ids, 4) || !aligned(grad_combine, 4))) || !aligned(loss, 4) ||
         !aligned(dlogits, 4))
         return DO_ERR_INVALID_ARG;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < dol::workspace_bytes(p, false))
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < dol::workspace_bytes(p))
         return DO_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
     char *ws = static_cast<char *>(workspace);
-    const dol::WsLayout w = dol::ws_layout_for(p, workspace_bytes, false);
+    const dol::WsLayout w = dol::ws_layout(p);
     int *status = reinterpret_cast<int *>(ws);
     int *done = reinterpret_cast<int *>(ws + w.done);
     uint8_t *idx = reinterpret_cast<uint8_t *>(ws + w.idx);
@@ -461,7 +472,7 @@ do_status do_routed_backward(const float *logits, int64_t T, int32_t E, int32_t 
     const bool local = d_scale == 1.0f;
     const bool have_idx = dol::signatures_fast_supported(logits, p);
     const bool alu = split_fast(p, logits, bits, D) && aligned(dlogits, 16);
-    const bool mma = split_mma(p, logits, w) && dol::loss_mma_supported(p, logits, dlogits) &&
+    const bool mma = split_mma(p, logits) && dol::loss_mma_supported(p, logits, dlogits) &&
                      !(alu && dol::loss_alu_faster(p, gate));
     unsigned char *bimg = reinterpret_cast<unsigned char *>(ws + w.bimg);
     cudaError_t e;

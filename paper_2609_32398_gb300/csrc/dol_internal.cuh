@@ -9,6 +9,8 @@
 
 #include <atomic>
 
+#include "doloss.h"
+
 namespace dol {
 
 constexpr unsigned kFull = 0xffffffffu;
@@ -81,20 +83,20 @@ struct WsLayout {
 constexpr int kMaxSigCtas = 255;
 int max_sig_ctas_per_problem(const Problem &p);
 // wide: with room for the co-occurrence triangles at every size that has them
-// (cooc_sizes_ok); without it only E in {32, 64, 128}, k in {1, 2, 4, 8} have
-// it and the other sizes take D from the signatures (a fixed scratch array
-// that is too small for the triangles still serves them).
-WsLayout ws_layout(const Problem &p, bool wide);
-inline size_t workspace_bytes(const Problem &p, bool wide = true) { return ws_layout(p, wide).total; }
+// (cooc_sizes_ok).  Without it (the library's fixed scratch array, where the wide
+// layout does not fit) only E in {32, 64, 128}, k in {1, 2, 4, 8} have it and the
+// other sizes take D from the signatures.
+WsLayout ws_layout(const Problem &p, bool wide = true);
+inline size_t workspace_bytes(const Problem &p) { return ws_layout(p).total; }
 // What a call without routing outputs needs: the layout up to the routing scratch.
 inline size_t workspace_bytes_plain(const Problem &p, bool wide = true) {
     return ws_layout(p, wide).route_base;
 }
-// The layout a call of `bytes` workspace uses.
-inline WsLayout ws_layout_for(const Problem &p, size_t bytes, bool plain) {
-    const WsLayout w = ws_layout(p, true);
-    return (plain ? w.route_base : w.total) <= bytes ? w : ws_layout(p, false);
-}
+// do_forward_backward on a workspace of the wide or the narrow layout (api.cu).
+do_status forward_backward_plain(const float *logits, int64_t T, int32_t E, int32_t k, int32_t L,
+                                 int32_t gate, float grad_scale, uint32_t *bits, int32_t *counts,
+                                 int32_t *D, float *loss, int64_t *origin_do, float *dlogits,
+                                 void *workspace, size_t workspace_bytes, void *stream, bool wide);
 
 // Partial-sum slots per problem that the workspace has at least (with W if that
 // is more).

@@ -128,8 +128,9 @@ extern "C" do_status do_forward_backward_static(const float *logits, int64_t T, 
     // kernel, the image of D' by the reduction kernel, every entry of it).
     char *base = static_cast<char *>(ws);
     if (cudaMemsetAsync(base, 0, dol::kWsHeader, s) != cudaSuccess) return DO_ERR_CUDA;
-    st = do_forward_backward(logits, T, E, k, L, gate, grad_scale, bits, counts, D, loss, origin_do,
-                             dlogits, ws, DO_STATIC_SCRATCH_BYTES, stream);
+    const bool wide = dol::workspace_bytes_plain(p) <= DO_STATIC_SCRATCH_BYTES;
+    st = dol::forward_backward_plain(logits, T, E, k, L, gate, grad_scale, bits, counts, D, loss,
+                                     origin_do, dlogits, ws, DO_STATIC_SCRATCH_BYTES, stream, wide);
     if (st != DO_OK) return st;
     if (status_flags &&
         cudaMemcpyAsync(status_flags, base, sizeof(int32_t), cudaMemcpyDeviceToDevice, s) !=

@@ -249,3 +249,26 @@ def test_binding_signatures_match_the_header(dl):
         want_args, want_res = dl.EXPORTS[name]
         assert args == want_args, (name, args, want_args)
         assert res == want_res, (name, res, want_res)
+
+
+@pytest.mark.parametrize("T,E,k,L", [(150000, 8, 2, 255), (262144, 96, 6, 1), (4096, 128, 8, 1), (1 << 20, 256, 8, 1),
+                                     (777, 33, 5, 2)])
+def test_workspace_sizes_are_required_in_full(dl, T, E, k, L):
+    """Each call takes what its size function says and nothing less: the routed
+    ones refuse do_workspace_size bytes, all of them a byte less than their own."""
+    lib = dl.lib()
+    fake = ctypes.c_void_p(0x10000)
+    WS = 6
+    plain, routed = lib.do_workspace_size(T, E, k, L), lib.do_routed_workspace_size(T, E, k, L)
+    assert plain < routed
+    for n in (plain, routed - 1):
+        assert lib.do_forward_backward_routed(fake, T, E, k, L, 0, 1.0, fake, fake, fake, fake, None, None, fake,
+                                              fake, None, None, None, fake, n, None) == WS
+        assert lib.do_routed_forward(fake, T, E, k, L, 0, fake, fake, fake, None, fake, fake, None, None, None,
+                                     fake, n, None) == WS
+        assert lib.do_routed_backward(fake, T, E, k, L, 0, 1.0, 1.0, fake, fake, fake, None, None, fake, fake,
+                                      fake, n, None) == WS
+    assert lib.do_forward_backward(fake, T, E, k, L, 0, 1.0, fake, fake, fake, fake, None, None, fake, plain - 1,
+                                   None) == WS
+    assert lib.do_loss_fwd_bwd(fake, fake, fake, T, E, k, L, 0, 1.0, 1.0, fake, None, None, fake, plain - 1,
+                               None) == WS
