@@ -349,10 +349,13 @@ loss_fast_kernel(const LossArgs a) {
             for (int e = 1; e < 16; ++e) mx = fmaxf(mx, zz[e]);
 #pragma unroll
             for (int o = G / 2; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, o));
-            const float mxs = mx * 1.4426950408889634f;
+            // 2^(z log2 e - max log2 e); beyond 2^22, where that difference would
+            // lose its fraction (or overflow), 2^((z - max) log2 e)
+            const float sh = fabsf(mx) < 4194304.0f ? 0.0f : mx;
+            const float mxs = (mx - sh) * 1.4426950408889634f;
 #pragma unroll
             for (int e = 0; e < 16; ++e) {
-                gv[e] = ex2_approx(fmaf(zz[e], 1.4426950408889634f, -mxs));
+                gv[e] = ex2_approx(fmaf(zz[e] - sh, 1.4426950408889634f, -mxs));
                 den += gv[e];
                 num = fmaf(gv[e], w[e], num);
             }

@@ -145,6 +145,42 @@ def test_low_logits(dl, T, E, k, shift):
     check_loss(z[0].numpy(), f, D, k, 0, float(loss[0]), dz[0], zmax=zmax)
 
 
+# the softmax gate far from zero: rows of the lowest value (uniform weights), rows and
+# whole boxes of masks of several sizes, large rows of either sign, ordinary rows
+# beside them; one to four boxes and the gather kernels
+@pytest.mark.parametrize("T,E,k", [(300, 24, 3), (300, 64, 5), (2300, 64, 8), (515, 96, 6), (515, 100, 8), (4100, 128, 8),
+                                   (300, 32, 4), (300, 200, 5), (300, 256, 8)])
+def test_softmax_far_from_zero(dl, T, E, k):
+    low = torch.finfo(torch.float32).min
+    z = workloads.random_logits(T, E, seed=T + E)
+    z[0, 1] = low
+    z[0, 2] = -1e9
+    z[0, 3, : E // 2] = 1e9
+    z[0, 4, E // 2:] = -1e10
+    z[0, 5, : E // 2] = -1e29
+    z[0, 6] += 2.9e6                                  # around the line where the form changes
+    z[0, 7] -= 4.3e6
+    z[0, 8, E // 2:] = low
+    z[0, 9, :] = low
+    z[0, 9, E - 1] = 0.0
+    z[0, 10] *= 1e12
+    z[0, 11, : E // 2] += 4194304.0
+    z[0, 12, E // 2:] -= 4194304.0
+    z[0, T - 1, 1:] = -3e38
+    zc = z.cuda()
+    out = dl.forward_backward(zc, k, workloads.GATE_SOFTMAX)
+    loss, _, dz = dl.loss_fwd_bwd(zc, out.bits, out.D, k, workloads.GATE_SOFTMAX)
+    torch.cuda.synchronize()
+    assert dl.device_status(out.workspace) == 0
+    zl = z[0].numpy()
+    f = oracle.select(zl, k)
+    D = oracle.hamming(f)
+    # logits that weigh anything are within 8 of their row's maximum, or at least 0.25
+    # apart and exact there: the arguments of the exponentials are as in the note above
+    check_loss(zl, f, D, k, workloads.GATE_SOFTMAX, float(out.loss[0]), out.dlogits[0])
+    check_loss(zl, f, D, k, workloads.GATE_SOFTMAX, float(loss[0]), dz[0])
+
+
 # one zeroed workspace for two shapes in turn, both orders, each also twice running:
 # nothing that a call leaves in it may reach the next one
 @pytest.mark.parametrize("one,two", [
