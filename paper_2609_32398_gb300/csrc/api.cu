@@ -249,17 +249,18 @@ do_status forward_backward_impl(const float *logits, int64_t T, int32_t E, int32
     const bool loss_idx = select && aligned(bits, 16) &&
                           (dol::loss_fast_supported(p, logits, D, dlogits) ||
                            dol::loss_fast256_supported(p, logits, D, dlogits));
-    const bool mma = select && w.image && dol::loss_mma_supported(p, logits, dlogits) &&
+    const bool cooc = w.cooc && dol::select_cooc_supported(logits, p, route);
+    const bool mma = cooc && w.image && dol::loss_mma_supported(p, logits, dlogits) &&
                      !(loss_idx && dol::loss_alu_faster(p, gate));
     // (the tensor-core one where it is cheap for the selection to write them)
     const bool use_idx = loss_idx && (!mma || dol::signatures_fast_supported(logits, p));
     uint8_t *idx = use_idx ? reinterpret_cast<uint8_t *>(ws + w.idx) : nullptr;
     // the router GEMM runs only in the fused fast path, without routing outputs
-    if (rin && !(loss_idx && w.cooc && !ra &&
+    if (rin && !(loss_idx && cooc && !ra &&
                  dol::router_supported(p, rin->H, rin->X, rin->Wr, logits)))
         return DO_ERR_UNSUPPORTED;
     cudaError_t e;
-    if (select && w.cooc) {
+    if (cooc) {
         // signatures + per-CTA co-occurrence counts -> reduction, which builds
         // D = n_i + n_j - 2 c_ij and writes D, the counts and origin_do
         uint32_t *parts = reinterpret_cast<uint32_t *>(ws + w.cooc_parts);
@@ -410,7 +411,7 @@ do_status do_routed_forward(const float *logits, int64_t T, int32_t E, int32_t k
     int *rscratch = reinterpret_cast<int *>(ws + w.route_base);
     const dol::RouteOut route = {expert_ids, combine, gate};
     cudaError_t e = cudaSuccess;
-    if (dol::select_supported(logits, p) && w.cooc) {
+    if (w.cooc && dol::select_cooc_supported(logits, p, route)) {
         int *done = reinterpret_cast<int *>(ws + w.done);
         uint32_t *parts = reinterpret_cast<uint32_t *>(ws + w.cooc_parts);
         const dol::ZeroSpans zero = {{done, reinterpret_cast<int *>(origin_do), nullptr},

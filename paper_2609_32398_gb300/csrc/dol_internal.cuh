@@ -137,6 +137,11 @@ cudaError_t launch_signatures_fast_routed(const float *logits, const Problem &p,
 bool select_supported(const float *logits, const Problem &p);
 cudaError_t launch_select(const float *logits, const Problem &p, const SelectOut &o, cudaStream_t s);
 int sig_ctas_per_problem(const Problem &p);
+// Whether launch_select's triangles are exact for `ctas` CTAs per problem: the
+// tensor-core accumulators of select.cuh hold 4 c_ab in fp32, exact to
+// c_ab = 2^24, so that no CTA may take more tokens (sig_fast.cuh counts integers).
+bool cooc_counts_exact(int64_t W, int ctas);
+bool select_cooc_supported(const float *logits, const Problem &p, const RouteOut &route);
 cudaError_t launch_add_distances(const int *D, int *D_sum, int64_t n, cudaStream_t s);
 cudaError_t launch_hamming_accumulate(const uint32_t *bits, const Problem &p, int *D, cudaStream_t s);
 cudaError_t launch_origin_do(const int *D, const Problem &p, long long *origin_do, cudaStream_t s);

@@ -37,6 +37,11 @@ cudaError_t dispatch_select(const CUtensorMap &map, const Problem &p, const SelA
     return run_select<16, kCooc>(map, p, args, ctas, s);
 }
 
+bool takes_sig_fast(const float *logits, const Problem &p, const RouteOut &route) {
+    const uintptr_t al = reinterpret_cast<uintptr_t>(route.ids) | reinterpret_cast<uintptr_t>(route.combine);
+    return signatures_fast_supported(logits, p) && (!route.ids || al % 16 == 0);
+}
+
 }  // namespace
 
 // One CTA per SM over all problems, at most one per tile.
@@ -57,17 +62,20 @@ bool select_supported(const float *logits, const Problem &p) {
            (int64_t)p.L * p.T + 32 < (int64_t)INT_MAX;
 }
 
+bool cooc_counts_exact(int64_t W, int ctas) { return 32 * ((W + ctas - 1) / ctas) <= (int64_t)1 << 24; }
+
+bool select_cooc_supported(const float *logits, const Problem &p, const RouteOut &route) {
+    return select_supported(logits, p) && cooc_sizes_ok(p.E, p.k) &&
+           (takes_sig_fast(logits, p, route) || cooc_counts_exact(p.W, sig_ctas_per_problem(p)));
+}
+
 cudaError_t launch_select(const float *logits, const Problem &p, const SelectOut &o, cudaStream_t s) {
-    if (signatures_fast_supported(logits, p)) {
-        if (!o.route.ids)
-            return launch_signatures_fast(logits, p, o.bits, o.counts, o.idx, o.cooc, o.zero, o.status, s);
-        if (reinterpret_cast<uintptr_t>(o.route.ids) % 16 == 0 &&
-            reinterpret_cast<uintptr_t>(o.route.combine) % 16 == 0)
-            return launch_signatures_fast_routed(logits, p, o.bits, o.counts, o.idx, o.cooc, o.zero,
-                                                 o.status, o.route, s);
-    }
+    if (takes_sig_fast(logits, p, o.route))
+        return o.route.ids ? launch_signatures_fast_routed(logits, p, o.bits, o.counts, o.idx, o.cooc, o.zero,
+                                                           o.status, o.route, s)
+                           : launch_signatures_fast(logits, p, o.bits, o.counts, o.idx, o.cooc, o.zero, o.status, s);
     CUtensorMap map;
-    if (!select_supported(logits, p) || (o.cooc && !cooc_sizes_ok(p.E, p.k)) || (o.idx && p.E > 256))
+    if (!select_supported(logits, p) || (o.cooc && !select_cooc_supported(logits, p, o.route)) || (o.idx && p.E > 256))
         return cudaErrorInvalidValue;
     // one copy per tile where the boxes of a row are whole and many (E = 256,
     // T = 2^20, 4 problems: the step 3,893 -> 3,808 us; at E = 128 a copy per

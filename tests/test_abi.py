@@ -272,3 +272,14 @@ def test_workspace_sizes_are_required_in_full(dl, T, E, k, L):
                                    None) == WS
     assert lib.do_loss_fwd_bwd(fake, fake, fake, T, E, k, L, 0, 1.0, 1.0, fake, None, None, fake, plain - 1,
                                None) == WS
+
+
+def test_tokens_of_a_cta_stay_exact_in_fp32_counts(dl):
+    """The selection kernel's fp32 co-occurrence counts hold 4 c exactly to c = 2^24:
+    problems with more tokens per CTA are counted from the signatures instead."""
+    exact = ctypes.CDLL(dl.LIB_PATH)._ZN3dol17cooc_counts_exactEli
+    exact.argtypes, exact.restype = [ctypes.c_int64, ctypes.c_int], ctypes.c_bool
+    words = (1 << 24) // 32
+    assert exact(1, 1) and exact(words, 1) and not exact(words + 1, 1)
+    assert exact(152 * words, 152) and not exact(152 * words + 1, 152)
+    assert not exact(20000000 // 32, 1)                  # 80 problems of 2e7 tokens, one CTA each
