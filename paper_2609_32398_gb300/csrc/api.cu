@@ -491,7 +491,9 @@ do_status do_routed_backward(const float *logits, int64_t T, int32_t E, int32_t 
                                      img_ok, local ? nullptr : D);
         if (rg_mma) return from_cuda(e);
     } else if (alu) {
-        e = dol::launch_idx_from_bits(bits, p, idx, nullptr, 0, s);
+        // the chosen experts: as the forward half left them, where it did
+        const bool left = have_idx && dol::cooc_counts_exact(p.W, dol::sig_ctas_per_problem(p));
+        e = left ? cudaSuccess : dol::launch_idx_from_bits(bits, p, idx, nullptr, 0, s);
         // the row sums of D come from the counts only for the local matrix
         if (e == cudaSuccess)
             e = dol::launch_loss_fast(logits, idx, D, local ? counts : nullptr, p, gate,

@@ -7,6 +7,8 @@ Tolerances: bits, counts, D, origin_do and the routing ids bit-exact; the
 loss within 1e-5 relative; dlogits within 1e-4 of the largest DO-gradient
 entry (the path's gradient tolerance) plus the routing gradient's
 per-entry bound (4k + 32) 2^-24 w (|g| + sum |g| w) (1 - s)."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -233,3 +235,32 @@ def test_global_do_binding_at_one_rank_is_the_local_step(dl):
     torch.cuda.synchronize()
     assert torch.equal(D, ref.D) and torch.equal(counts, ref.counts)
     assert torch.equal(loss, ref.loss) and torch.equal(dz, ref.dlogits)
+
+
+def launches(fn):
+    """Stream operations of one call, counted as the nodes of its capture."""
+    drv = ctypes.CDLL("libcuda.so.1")
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        fn()
+        s.synchronize()
+        st, g, n = ctypes.c_void_p(s.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t(0)
+        assert drv.cuStreamBeginCapture_v2(st, 2) == 0          # relaxed
+        fn()
+        assert drv.cuStreamEndCapture(st, ctypes.byref(g)) == 0
+        assert drv.cuGraphGetNodes(g, None, ctypes.byref(n)) == 0
+        drv.cuGraphDestroy(g)
+    return n.value
+
+
+@pytest.mark.parametrize("T,E,k,gate,n", [
+    (2000, 64, 8, 0, 2), (500, 32, 8, 0, 2), (4000, 128, 8, 1, 2), (70000, 128, 2, 0, 2),   # gather, routing gradient
+    (4000, 128, 8, 0, 1), (3000, 96, 6, 0, 2)])                  # tensor cores, with and without the gradient inside
+def test_backward_half_launches(dl, T, E, k, gate, n):
+    """The backward half reads the chosen experts that the forward half left:
+    the loss kernel and, where that does not add it, the routing gradient's."""
+    z = workloads.random_logits(T, E, seed=T).cuda()
+    out, r = dl.routed_forward(z, k, gate)
+    g = torch.randn(1, T, k, device="cuda")
+    assert launches(lambda: dl.routed_backward(z, r.expert_ids, g, k, gate, out=out)) == n
+    assert dl.device_status(out.workspace) == 0
