@@ -12,8 +12,8 @@ one ex2.approx (2 ulp) of a product rounded at |z| <= 8 (12 u) and one rcp.appro
 (1 ulp), so s, the sums and their quotient are within (E + 64) u; the integers
 behind w are exact below 2^24 and rounded once above.  So
   |dz - ref| <= 2 (E + 64) u p (1 - s) (|w| + M_t),  |loss - ref| <= 2 (E + 64) u sum_t M_t,
-the factor 2 for the two factors of the product (at E <= 64 and in the gather kernel
-1 - s comes as s - s^2, within u / (1 - s) <= 150 u at z <= 5, inside the same bound).  u p_max max|w| is added for
+the factor 2 for the two factors of the product (in the gather kernels 1 - s comes
+as s - s^2, within u / (1 - s) <= 150 u at z <= 5, inside the same bound).  u p_max max|w| is added for
 results rounded near zero.  Where |z| goes beyond 8 the rounded product z log2 e and
 the rounded log2 e put up to 1.25 |z| u more into each s, and so on into every sum:
 E + 64 + 1.25 (|z| - 8) in the place of E + 64.
@@ -39,7 +39,8 @@ def dl():
     return m
 
 
-def check_loss(z, f, D, k, gate, loss, dz, d_scale=1.0, extra=0.0, extra_bound=0.0, zmax=8.0):
+def check_loss(z, f, D, k, gate, loss, dz, d_scale=1.0, extra=0.0, extra_bound=0.0, zmax=8.0,
+               near_zero=True):
     T, E = z.shape
     p = oracle.gate(z, gate)
     w = oracle.dloss_dp(D, f, T, k, d_scale)
@@ -50,7 +51,7 @@ def check_loss(z, f, D, k, gate, loss, dz, d_scale=1.0, extra=0.0, extra_bound=0
     if dz is None:
         return
     oms = 1.0 if gate == workloads.GATE_SOFTMAX else 1.0 / (1.0 + np.exp(z.astype(np.float64)))
-    bound = tol * p * oms * (np.abs(w) + M) + U * p.max() * np.abs(w).max()
+    bound = tol * p * oms * (np.abs(w) + M) + near_zero * U * p.max() * np.abs(w).max()
     err = np.abs(dz.double().cpu().numpy() - oracle.gate_backward(z, w, gate) - extra)
     bound = bound + extra_bound
     assert (err <= bound).all(), ("dlogits", float((err / bound).max()))
@@ -143,6 +144,20 @@ def test_low_logits(dl, T, E, k, shift):
     zmax = float(z.abs().max())
     check_loss(z[0].numpy(), f, D, k, 0, float(out.loss[0]), out.dlogits[0], zmax=zmax)
     check_loss(z[0].numpy(), f, D, k, 0, float(loss[0]), dz[0], zmax=zmax)
+
+
+# saturated experts: 1 - s keeps its relative accuracy where s is one to rounding, at
+# every number of boxes (the bound without its term for results near zero)
+@pytest.mark.parametrize("T,E,k", [(515, 32, 3), (515, 64, 5), (5000, 64, 8), (515, 96, 6), (515, 128, 8)])
+def test_saturated_experts(dl, T, E, k):
+    z = workloads.random_logits(T, E, seed=T + E)
+    z[0, :, : E // 2] += 20.0
+    out = dl.forward_backward(z.cuda(), k)
+    torch.cuda.synchronize()
+    assert dl.device_status(out.workspace) == 0
+    f = oracle.select(z[0].numpy(), k)
+    check_loss(z[0].numpy(), f, oracle.hamming(f), k, 0, float(out.loss[0]), out.dlogits[0],
+               zmax=float(z.abs().max()), near_zero=False)
 
 
 # the softmax gate far from zero: rows of the lowest value (uniform weights), rows and
