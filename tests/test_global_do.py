@@ -157,7 +157,7 @@ def test_two_gloo_ranks_on_the_gpu_path():
     none of the kernels waits on another rank) each hold half of the c3
     tokens.  The summed D is the oracle's matrix of all tokens, and each
     rank's loss and gradient are the oracle's for its shard with d_scale = 1/2
-    (the ALU loss kernel)."""
+    (the tensor-core kernel on the image of the summed matrix)."""
     import oracle
     from paper_2609_32398_gb300 import workloads
 
@@ -204,14 +204,16 @@ def test_window_of_one_micro_batch_is_the_local_step():
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("with_route", [False, True])
-def test_summed_matrix_beyond_the_fp16_image_takes_the_alu_kernel(with_route):
+@pytest.mark.parametrize("with_route,fold", [(False, 256), (True, 256), (False, 12000), (True, 12000)])
+def test_summed_matrix_beyond_the_fp16_image_is_gathered(with_route, fold):
     """Eq. global_do with a given matrix at E = 128, two problems in one call:
     problem 0's matrix (three local matrices' sum) fits the two fp16 pieces of
-    the tensor-core kernel's image of D', problem 1's (a 256-fold sum, row sums
-    above 2^23) does not and goes to the ALU kernel.  Both problems' loss and
-    gradient equal the oracle's for their matrix, with d_scale = 1/3, with and
-    without the combine weights' gradient added in the same call."""
+    the tensor-core kernel's image of D'; problem 1's fits with the marker
+    diagonal (a 256-fold sum, row sums above 2^23), or has entries of 2^22 and
+    more (a 12000-fold sum) and its rows are gathered from it in the same launch.
+    Both problems' loss and gradient equal the oracle's for their matrix, with
+    d_scale = 1/3, with and without the combine weights' gradient added in the
+    same call."""
     import oracle
     import paper_2609_32398_gb300.doloss as dl
     from paper_2609_32398_gb300 import workloads
@@ -222,9 +224,10 @@ def test_summed_matrix_beyond_the_fp16_image_takes_the_alu_kernel(with_route):
     out, route = dl.routed_forward(zc, k, 0, with_routing=with_route)
     torch.cuda.synchronize()
     D_loc = [oracle.hamming(oracle.select(z[l].numpy(), k)) for l in range(L)]
-    mult = (3, 256)
+    mult = (3, fold)
     D_sum = np.stack([D_loc[l].astype(np.int64) * mult[l] for l in range(L)])
     assert D_sum[1].sum(axis=1).max() >= 1 << 23 > D_sum[0].sum(axis=1).max()
+    assert (D_sum[1].max() >= 1 << 22) == (fold == 12000) and D_sum[1].sum(axis=1).max() < 1 << 31
     Dg = torch.from_numpy(D_sum.astype(np.int32)).cuda()
     gq = None
     if with_route:

@@ -272,15 +272,18 @@ def test_repeated_calls_reuse_workspace(dl):
                                    (66052, 8, 1), (128 * 5 + 1, 8, 2)])
 def test_tcgen05_and_alu_loss_kernels_agree(dl, T, k, L):
     """The fused call's gradient pass at E = 128 (V = F D' on the tensor cores)
-    against the split entry points, whose loss kernel gathers rows of D on the
-    ALU, and both against the oracle at small T."""
+    against the split entry points on logits that are not 16-byte aligned, which
+    only the kernels that gather rows of D on the ALU take, and both against the
+    oracle at small T."""
     z = workloads.random_logits(T, 128, L=L, seed=T + k, ties=T < 2000)
     out = gpu_run(dl, z, k, workloads.GATE_SIGMOID_NORM, grad_scale=2.0)
-    zc = z.cuda()
+    zc = torch.empty(z.numel() + 1, device="cuda")[1:].view(z.shape)
+    zc.copy_(z)
+    assert zc.data_ptr() % 16 != 0
     bits, counts = dl.signatures(zc, k)
     D = dl.pairwise_hamming(bits, T)
     loss, origin, dz = dl.loss_fwd_bwd(zc, bits, D, k, workloads.GATE_SIGMOID_NORM,
-                                       grad_scale=2.0)
+                                       grad_scale=2.0, dlogits=torch.empty(z.shape, device="cuda"))
     torch.cuda.synchronize()
     for a, b, name in ((out.bits, bits, "bits"), (out.counts, counts, "counts"), (out.D, D, "D"),
                        (out.origin_do, origin, "origin_do")):
@@ -347,20 +350,21 @@ def test_autograd_wrapper_gives_the_path_gradient(dl):
     assert torch.allclose(y.grad, 0.3 * ref.dlogits[0], rtol=1e-6, atol=0)
 
 
-def test_first_size_past_the_tensor_core_limit(dl):
+def test_first_size_of_the_marker_diagonal(dl):
     """T = 66053 at E = 128: (E - 1) T reaches 2^23, where the two-piece fp16
-    split of D' stops being exact, so the fused path takes the ALU gradient
-    pass; it must still match the oracle."""
+    split stops holding the diagonal of D', so that the tensor-core pass puts a
+    marker in its place; it must still match the oracle."""
     T, E, k = 66053, 128, 8
     z = workloads.random_logits(T, E, seed=66053)
     out = gpu_run(dl, z, k, 0)
     assert_layer(out, 0, z[0].numpy(), k, 0)
 
 
-@pytest.mark.parametrize("T,E,k", [(32, 32, 2), (1, 8, 2)])
+@pytest.mark.parametrize("T,E,k", [(32, 32, 2), (1, 8, 2), (1, 9, 2)])
 def test_largest_batch_of_problems(dl, T, E, k):
-    """L = 65535 problems in one call (the grid's y/z limit): the fast kernels
-    (E = 32) and the generic ones (E = 8), sampled layers against the oracle."""
+    """L = 65535 problems in one call (the grid's y/z limit): the two selection
+    kernels with triangles (E = 32, 8) and the generic one (E = 9), sampled layers
+    against the oracle."""
     L = 65535
     z = workloads.random_logits(T, E, L=L, seed=L + E)
     out = gpu_run(dl, z, k, 0)

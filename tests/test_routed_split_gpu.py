@@ -157,11 +157,10 @@ def test_bad_ids_are_reported(dl, T, E, k, gate):
 
 
 def test_split_with_unaligned_routing_outputs_and_no_dispatch(dl):
-    """expert_ids and combine 4- but not 16-byte aligned (the routing outputs
-    then come from the generic selection beside the fused path's) and no
-    dispatch arrays (the counts accumulator is then cleared by a memset):
-    the same outputs as the aligned call (the weights to their tolerance),
-    twice in a row."""
+    """expert_ids and combine 4- but not 16-byte aligned (the selection by
+    sorting networks then writes them, not the argmax kernel) and no dispatch
+    arrays: the same outputs as the aligned call (the weights to their
+    tolerance), twice in a row."""
     T, E, k, gate = 4096 + 33, 128, 8, 0
     z = workloads.random_logits(T, E, seed=17, ties=True).cuda()
     grad = torch.randn(1, T, k, device="cuda")
@@ -176,7 +175,7 @@ def test_split_with_unaligned_routing_outputs_and_no_dispatch(dl):
         dl.routed_forward(z, k, gate, out=out, route=route)
         torch.cuda.synchronize()
         assert torch.equal(route.expert_ids, ref_route.expert_ids)
-        # the generic selection kernel sums the weights in another order:
+        # the network selection sums the weights in another order:
         # both are within 2(k + 12) 2^-24 of the exact ratio
         assert (route.combine - ref_route.combine).abs().max() <= 4 * (k + 12) * 2.0 ** -24
         assert torch.equal(out.counts, ref_out.counts) and torch.equal(out.D, ref_out.D)
@@ -190,9 +189,9 @@ def test_split_with_unaligned_routing_outputs_and_no_dispatch(dl):
 
 
 @pytest.mark.parametrize("T,E,k,gate,routed", [
-    (4096 + 33, 128, 8, 0, True),     # ALU loss kernel with a summed D (no tensor-core image)
+    (4096 + 33, 128, 8, 0, True),     # tensor-core kernel, the image of the summed D built for it
     (4096 + 33, 128, 8, 0, False),
-    (2048, 64, 4, 1, True),
+    (2048, 64, 4, 1, True),           # ALU gather
     (999, 33, 3, 0, True),            # generic kernels
 ])
 def test_backward_half_with_a_summed_matrix(dl, T, E, k, gate, routed):

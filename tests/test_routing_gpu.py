@@ -57,7 +57,8 @@ def run_routing(dl, z_cpu, k, gate, **kw):
     return route
 
 
-# fast kernel: E in {32, 64, 128}, k in {1, 2, 4, 8}; generic kernel otherwise
+# argmax kernel: E in {32, 64, 128}, k in {1, 2, 4, 8}; sorting networks: other E that
+# are multiples of 4 up to 512, k <= 16; generic kernel otherwise
 @pytest.mark.parametrize("T,E,k,L,gate,ties", [
     (4096 + 33, 128, 8, 1, 0, False),
     (4096 + 33, 128, 8, 2, 1, True),
@@ -66,7 +67,7 @@ def run_routing(dl, z_cpu, k, gate, **kw):
     (77, 128, 1, 2, 0, True),
     (1, 128, 8, 1, 0, False),
     (2500, 33, 5, 2, 0, True),       # generic
-    (640, 256, 8, 1, 1, False),      # generic
+    (640, 256, 8, 1, 1, False),      # networks
     (97, 16, 16, 1, 0, True),        # k = E
     (500, 130, 100, 1, 0, True),     # one signature word per dispatch chunk
 ])
@@ -96,7 +97,7 @@ def test_routing_far_from_zero(dl, shift, gate):
     check_layer(route, 0, z[0].numpy(), 8, gate, 128)
 
 
-def test_unaligned_outputs_take_the_generic_kernel(dl):
+def test_unaligned_outputs_take_the_network_kernel(dl):
     """expert_ids and combine 4- but not 16-byte aligned: same results."""
     T, E, k = 2000, 128, 8
     z = workloads.random_logits(T, E, seed=9, ties=True)
