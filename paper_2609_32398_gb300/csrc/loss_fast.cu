@@ -43,6 +43,7 @@
 
 #include "dol_internal.cuh"
 #include "tma.cuh"
+#include "topk_net.cuh"
 
 namespace dol {
 namespace {
@@ -455,22 +456,13 @@ idx_from_bits_kernel(const uint32_t *__restrict__ bits, int64_t T, int64_t W, in
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const uint32_t lo_mask[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
     for (int64_t tile = wid; tile < ntiles; tile += nw) {
         const int64_t layer = tile / W, w = tile - layer * W;
         uint32_t m[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            uint32_t x = __ldg(bits + (layer * E + 32 * r + lane) * W + w);
-            // lane = expert column -> lane = token row (the same bit transpose)
-#pragma unroll
-            for (int s = 0; s < 5; ++s) {
-                const int j = 16 >> s;
-                const uint32_t lo = lo_mask[s];
-                const uint32_t p = __shfl_xor_sync(kFull, x, j);
-                x = (lane & j) ? ((x & ~lo) | ((p >> j) & lo)) : ((x & lo) | ((p << j) & ~lo));
-            }
-            m[r] = x;
+            // lane = expert column -> lane = token row
+            m[r] = transpose32_bits(__ldg(bits + (layer * E + 32 * r + lane) * W + w), lane);
         }
         const int64_t t = 32 * w + lane;
         if (t >= T) continue;
