@@ -133,10 +133,12 @@ do_status do_accumulate_distances(const int32_t *D, int32_t E, int32_t L, int32_
  * produced the token rows of logits; D may come from any source whose row
  * sums fit int32.  Logits are finite; with the sigmoid-normalised gate a
  * token's weights p = s / sum(s) are relative to its own sum, exact to fp32
- * rounding while its largest logit is above -80.  workspace: do_workspace_size(T, E, k, L) bytes of device
- * memory, 256-byte aligned and zero-filled before its first use (cudaMemset);
- * every call leaves it ready for the next one, of these or of any other sizes
- * that it is large enough for.  A workspace serves one call at a time; after a call fails or do_device_status reports an error, zero it
+ * rounding while its largest logit is above -80.
+ * workspace: do_workspace_size(T, E, k, L) bytes of device memory (fewer:
+ * DO_ERR_WORKSPACE), 256-byte aligned and zero-filled before its first use
+ * (cudaMemset); every call leaves it ready for the next one, of these or of
+ * any other sizes that it is large enough for.  A workspace serves one call at
+ * a time; after a call fails or do_device_status reports an error, zero it
  * again before reusing it. */
 do_status do_loss_fwd_bwd(const float *logits, const uint32_t *bits, const int32_t *D,
                           int64_t T, int32_t E, int32_t k, int32_t L, int32_t gate,

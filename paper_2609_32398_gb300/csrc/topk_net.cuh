@@ -187,8 +187,8 @@ __device__ __forceinline__ float topk_bound(uint32_t (&top)[KP], const uint32_t 
 // experts in ascending order.  Two passes without data-dependent branches or
 // addresses (see topk_lists and select.cuh), then the drop of the candidates
 // that share the k-th value's fp16 image beyond k, a row at a time by the whole
-// warp.  About 1,300 instructions a tile of 32 tokens at E = 128, K = 8, where
-// K rounds of an argmax over 16 group maxima took 2,800.
+// warp.  (The router step at T = 32768, H = 2048 takes 129.6 us with it against
+// 130.3 with K rounds of an argmax over 16 group maxima.)
 template <int NB, int K>
 __device__ __forceinline__ void select_net(unsigned char *tile, int lane, bool valid, int (&sel)[K]) {
     constexpr int KP = K <= 4 ? 4 : K;
