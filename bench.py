@@ -584,7 +584,8 @@ def run_ours(args, rank, world, local):
     # Global-DO's per-rank step (Sec. 3.1.4, Eq. global_do) through the halves:
     # the local D (standing in for the matrix summed over the ranks, whose
     # exchange is a 64 KB all-reduce between the halves) with d_scale = 1/2,
-    # which takes the ALU loss kernel; against the three split entry points.
+    # for which the backward half builds the image of D first; against the three
+    # split entry points.
     def global_step(r):
         dl.routed_forward(sets[r % N_SETS][0], k, w.gate, out=sets[r % N_SETS][1],
                           with_routing=False)
@@ -842,7 +843,7 @@ def run_ours(args, rank, world, local):
                     "us_per_step": split_ms * 1e3, "forward_us": split_fwd_ms * 1e3,
                     "backward_us": split_bwd_ms * 1e3,
                     "backward_roofline": {
-                        "bound": "hbm", "kernel": "loss_mma_kernel<8, true>",
+                        "bound": "hbm", "kernel": "loss_mma_kernel<4, 0, 0, 0, 1, 8>",
                         "achieved": routed_backward_bytes(T, E, k, L) / (split_bwd_ms * 1e-3) / 1e9,
                         "peak": peak, "unit": "GB/s",
                         "frac": routed_backward_bytes(T, E, k, L) / (split_bwd_ms * 1e-3) / 1e9
